@@ -1,0 +1,40 @@
+"""GPU parity of the C store and its rounding on the row tilings where they can go wrong:
+tiles of 0, 1 and 2 rows, tiles that end one row before, at and after a warp's 32 rows, a
+last row block of a few rows, columns of several tiles in one 32-column block. Each
+element type, with and without alpha and beta, in both kernel forms and through the
+split-k reduction; bit for bit against the split oracle."""
+
+import numpy as np
+import pytest
+
+import bsmm_gen as G
+import paper_1504_05046_gb300 as P
+from test_gpu_split_complex import run_c
+from test_gpu_split_f32 import run_f32
+from test_gpu_split import check
+
+pytestmark = pytest.mark.gpu
+
+ROWS = [0, 1, 2, 0, 28, 1, 33, 31, 32, 0, 64, 7, 3]  # 202 rows: boundaries at 31, 32, 65, 96, 128, 192
+COLS = [5, 0, 1, 26, 33, 2]
+
+
+def _problem(alpha, beta):
+    rng = np.random.default_rng(5)
+    r, c, q = (np.asarray(x, np.int32) for x in (ROWS, COLS, [17, 40, 3]))
+    am = (rng.random((len(r), len(q))) < 0.7).astype(np.uint8)
+    bm = (rng.random((len(q), len(c))) < 0.7).astype(np.uint8)
+    return G._assemble("store", r, c, q, am, bm, rng, "uniform", "store", alpha, beta)
+
+
+@pytest.mark.parametrize("form", [dict(store_warps=2), dict(store_warps=1), dict(ksplit=2)])
+@pytest.mark.parametrize("alpha,beta", [(1.0, 0.0), (-0.5, 0.0), (1.0, 0.75), (0.375, -2.0)])
+@pytest.mark.parametrize("elem", ["f64", "f32", "c128"])
+def test_row_segments(elem, alpha, beta, form):
+    prob = _problem(alpha, beta)
+    if elem == "f64":
+        check(prob, 6, **form)
+    elif elem == "f32":
+        run_f32(G.as_float32(prob), **form)
+    else:
+        run_c(G.as_complex(prob, 3), **form)
