@@ -215,6 +215,18 @@ __device__ __forceinline__ void tmem_zero8(uint32_t taddr) {
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// One lane of a converged warp. Code that a whole warp runs up to this choice keeps its
+// addresses and descriptors in uniform registers, which tcgen05.mma takes them from.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(r));
+  return r != 0;
+}
+
 // Shared-memory matrix descriptor: K-major operand, 64-byte swizzle, 8-row groups of
 // 64-byte rows (stride between 8-row groups = 512 bytes).
 __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
@@ -1245,11 +1257,14 @@ struct GroupRule {
 // then every MMA warp's commit marks the buffer full once its MMAs have finished.
 __device__ __forceinline__ void close_group(bool first, int4* gdesc, uint64_t* gready, uint64_t* tfull, uint32_t buf,
                                             int gk0, const GroupRule& grp, bool last) {
-  if (first) {
-    gdesc[buf] = make_int4(gk0, grp.sig, (grp.uni ? 1 : 0) | (last ? 2 : 0), 0);
-    mbar_arrive(&gready[buf]);
+  if (elect_one()) {
+    if (first) {
+      gdesc[buf] = make_int4(gk0, grp.sig, (grp.uni ? 1 : 0) | (last ? 2 : 0), 0);
+      mbar_arrive(&gready[buf]);
+    }
+    umma_commit(&tfull[buf]);
   }
-  umma_commit(&tfull[buf]);
+  __syncwarp();
 }
 
 // The values of one own k block of a unit's list that the MMA warps need, loaded ahead.
@@ -1437,7 +1452,10 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
     // products; all of them accumulate (the epilogue zeroes a buffer once drained), and
     // the order in which the tensor core applies them does not matter: every partial sum
     // is an integer below 2^24, exact in FP32.
-    if (lane == 0) {
+    // The whole warp walks the list and one elected lane issues: every partial product's
+    // descriptors then come from uniform registers. (With lane 0 alone in the loop each had
+    // to be moved there first: 837 against 753 cycles per 6-slice chunk, issue alone.)
+    {
       const int mw = warp - 1;
       int stage = 0;
       uint32_t phase = 0;
@@ -1489,7 +1507,7 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
             buf = tcount & 1;
             const uint32_t use = tcount >> 1;
             // the buffer was drained and zeroed by the epilogue (use 0: zeroed at start)
-            if (!wait1(&tempty[buf], use & 1, abort_flag, a.err)) {
+            if (!wait_warp(&tempty[buf], use & 1, abort_flag, a.err)) {
               ok = false;
               in_group = false;
               break;
@@ -1507,7 +1525,7 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
                 close_group(mw == 0, gdesc, gready, tfull, buf, gk0, grp, false);
                 tcount++;
                 buf = tcount & 1;
-                if (!wait1(&tempty[buf], (tcount >> 1) & 1, abort_flag, a.err)) {
+                if (!wait_warp(&tempty[buf], (tcount >> 1) & 1, abort_flag, a.err)) {
                   ok = false;
                   break;
                 }
@@ -1515,12 +1533,12 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
                 dbase = tmem_base + buf * BUF_COLS;
               }
             }
-            if (!wait1(&full[stage], phase, abort_flag, a.err)) {
+            if (!wait_warp(&full[stage], phase, abort_flag, a.err)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            {
+            if (elect_one()) {
               const uint64_t soff = (uint64_t)((stage * STAGE) >> 4);
               const uint64_t ad = adesc0 + soff, bd = bdesc0 + soff;
               const bool two = q - kc * kSplitKC > 16;  // second 16-deep step of the 32-deep chunk
@@ -1530,8 +1548,9 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
                 umma_f16(dbase + dcol[j], ad + aoff[j], bd, idp[j], 1u);
                 if (two) umma_f16(dbase + dcol[j], ad + aoff[j] + 2, bd + 2, idp[j], 1u);
               }
+              umma_commit(&empty[stage]);  // the stage is free once these MMAs have finished
             }
-            umma_commit(&empty[stage]);  // the stage is free once these MMAs have finished
+            __syncwarp();
             any = true;
             if (++stage == stages) {
               stage = 0;
@@ -1549,13 +1568,14 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
           tcount++;
         }
       }
-      // drain: every MMA this thread issued has completed before TMEM is released
+      // drain: every MMA this warp issued has completed before TMEM is released
       if (any) {
-        umma_commit(&drain[mw]);
+        if (elect_one()) umma_commit(&drain[mw]);
+        __syncwarp();
         const int64_t t0 = gtimer();
         while (!mbar_try_wait(&drain[mw], 0)) {
           if (gtimer() - t0 > kWaitNs) {
-            atomicOr(a.err, kErrTimeout);
+            if (lane == 0) atomicOr(a.err, kErrTimeout);
             break;
           }
         }
