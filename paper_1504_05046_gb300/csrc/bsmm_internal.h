@@ -163,6 +163,7 @@ struct SplitArgs {
   // Mtot, and padded like a colexp row), the parts of the accumulator unit 2^L
   int32_t* emaxr;
   int32_t* emaxc;
+  int32_t qmax;             // the largest inner block
   int32_t kdepth;           // deepest exact FP32 accumulation (inner elements) for s slices
   int32_t transa, transb;   // transposed operand storage (bsmm_options)
   // per-row / per-column scaling (split_scale = 1): exponents of every row of every A tile
@@ -303,6 +304,7 @@ struct bsmm_plan_s {
   int s = 0, tn = 0, stages = 0, RB = 0, CB = 0, kwords = 0, cl = 1, CBG = 0;
   int sw = 0;                // contraction kernel with C store warps
   int epi_walk = 0;          // the epilogue walks the k lists itself (SplitArgs::epi_walk)
+  int32_t qmax = 0;          // the largest inner block
   int deep = 0;              // some inner block is deeper than the exact FP32 depth
   int64_t Mtot = 0, Ntot = 0, colexp_ld = 0;
   int64_t apk_bytes = 0, bpk_bytes = 0;

@@ -86,6 +86,7 @@ void fill_split_args(bsmm_plan_s* p, SplitArgs& a, double alpha, const void* A, 
   a.coladj = (int16_t*)p->d_coladj.p;
   a.emaxr = (int32_t*)p->d_emaxr.p;
   a.emaxc = (int32_t*)p->d_emaxc.p;
+  a.qmax = p->qmax;
   a.kdepth = split_max_depth(p->s);
   a.transa = p->opt.transa;
   a.transb = p->opt.transb;

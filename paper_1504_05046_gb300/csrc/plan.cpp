@@ -429,8 +429,10 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   {
     int64_t depth = 0;
     p->deep = 0;
+    p->qmax = 0;
     for (int k = 0; k < K; k++) {
       depth += p->q[k];
+      p->qmax = std::max(p->qmax, p->q[k]);
       if (p->q[k] > maxd) p->deep = 1;
     }
     if (depth > kSplitMaxInner) {

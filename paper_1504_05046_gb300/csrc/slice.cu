@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 #include <type_traits>
@@ -14,8 +15,6 @@
 namespace bsmm {
 
 namespace {
-
-constexpr int kAChunk = kSplitBM * kSplitKC * 2;  // bytes of one slice of a 128x32 A chunk
 
 // byte offset of element (row, k) inside one 64-byte-swizzled chunk slice (rows of 32 elements)
 __device__ __forceinline__ uint32_t swz64(int row, int k) {
@@ -380,112 +379,235 @@ __global__ void __launch_bounds__(256) split_class_kernel(SplitArgs a) {
 }
 
 // ---------------------------------------------------------------- kernel 2: slices
-// Slice 8 consecutive inner elements (one 16-byte chunk of a swizzled row) of one
-// packed row and store the s chunks.
 // The slicing recurrence N_t = rint(rho_{t-1} 2^(7t)), rho_t = rho_{t-1} - N_t 2^(-7t)
 // telescopes: with Z_t = sum_{u<=t} N_u 2^(7(t-u)) one has Z_t = rint(x 2^(7t-e)) (the
 // subtracted 128 Z_{t-1} is even, so round-half-even commutes with it), hence
-// N_t = Z_t - 128 Z_{t-1}. Each Z_t is computed exactly from the mantissa with integer
-// shifts and a round-half-even step; no floating-point operation is involved.
-// All Z_t of one element come from one window of its significand: x 2^-e = +-m 2^ex with
-// an integer m < 2^53; at the finest level t = S the window is W = floor(m 2^-k),
-// k = -(ex + 7S), with the round bit R (bit k-1 of m) and the sticky flag (any lower bit
-// set); level t < S drops a = 7(S-t) more bits of W, rounding with bit a-1 of W and the
-// bits below it (the finest level's fraction included). The window's shifts are
-// compile-time constants. Only the low 32 bits of Z_t are kept: N_t is small, so
-// Z_t - 128 Z_(t-1) is exact in 32-bit wrap-around arithmetic.
-struct SliceWindow {
-  unsigned long long W;  // floor(m 2^-k)
-  bool R, T, F;          // round bit and sticky bits at the finest level; F = any bit below W
-  __device__ __forceinline__ void init(unsigned long long m, int k) {
-    if (k <= 0) {  // exact (a subnormal tile's elements, or a non-finite input already reported)
-      W = -k >= 63 ? 0ull : m << -k;
-      R = T = F = false;
-    } else if (k >= 64) {
-      W = 0ull;
-      R = false;
-      T = F = m != 0ull;
-    } else {
-      W = m >> k;
-      R = (m >> (k - 1)) & 1ull;
-      T = (m & ((1ull << (k - 1)) - 1ull)) != 0ull;
-      F = R || T;
-    }
+// N_t = Z_t - 128 Z_{t-1}. The signs of Z_t and N_t are x's and -x's alike (half-even is
+// symmetric), so magnitudes are sliced and the sign is multiplied in at the end.
+//
+// Window. V = floor(|x| 2^(7S-e+2)): |x| in units of 2^-2 of the finest slice's unit. Level
+// t's unit is then 2^p with p = 2 + 7(S-t), and Z_t = floor((V + 2^(p-1)) / 2^p), except
+// that an exact tie has to go to the even quotient. x is at a tie of level t exactly when
+// no bit below V is set and V's lowest set bit is bit p-1, so it is at a tie of at most one
+// level, and there V +- 1 (up when bit p, the quotient's last bit, is set) rounds as
+// half-even asks without changing any other level's rounding. A tie needs V even and
+// nothing below it, which a thread tests for its 8 elements at once: seldom true of doubles
+// of full mantissa, always of float32 and integer data.
+//
+// Digits. With r_t = (V + 2^(p-1)) mod 2^p = (V mod 2^p) ^ 2^(p-1), what rounding at level
+// t leaves over (biased), N_t 2^p = r_{t-1} - r_t + 2^(p-1) - 2^(p+6). So a digit takes one
+// three-input logic instruction (r_t) and one three-input addition, which also adds the
+// bits of 2^23: the sum read as a float is 2^23 + (N_t + 64) 2^p, one multiply-add from
+// N_t. The multiply-add, the sign and the packing run beside the integer pipe. Three
+// levels fit a 32-bit word (p = 2, 9, 16); the next three are those of V >> 21, whose
+// dropped bits are the same in both remainders.
+//
+// What bounds it: HBM (8 bytes read and 2S written per element): 16384 dense, six slices,
+// 10.7 GB in 1.96 ms (5.5 TB/s), where significand windows with variable rounding per level
+// took 2.92 ms (integer pipe 80% busy, DRAM 43%, and each block's chunks one after the
+// other with nothing in flight between them). float32 8192, four slices: 0.62 to 0.45 ms.
+template <typename T>
+struct Slice2;  // two slices' values in one word; times the elements' signs
+template <>
+struct Slice2<__nv_bfloat16> {
+  static constexpr uint32_t kOnes = 0x3F803F80u;
+  __device__ static uint32_t pack(float lo, float hi) {  // <= 8 significant bits: truncation is exact
+    return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
   }
-  // low 32 bits of Z at the level a bits coarser than the finest. For A > 0 the rounding
-  // is one addition: with h = 2^(A-1) and b = (bit A of W) | F, W + h - 1 + b carries into
-  // bit A exactly when the dropped part exceeds h, or equals h with an odd quotient or a
-  // nonzero fraction below W (round half to even).
-  template <int A>
-  __device__ __forceinline__ uint32_t z() const {
-    if constexpr (A == 0) {
-      return (uint32_t)W + ((R && (T || (W & 1ull))) ? 1u : 0u);
-    } else {
-      const unsigned long long b = ((W >> A) & 1ull) | (F ? 1ull : 0ull);
-      return (uint32_t)((W + ((1ull << (A - 1)) - 1ull) + b) >> A);
-    }
+  __device__ static uint32_t mul(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 r = __hmul2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&r);
+  }
+};
+template <>
+struct Slice2<__half> {
+  static constexpr uint32_t kOnes = 0x3C003C00u;
+  __device__ static uint32_t pack(float lo, float hi) {
+    const __half2 r = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&r);
+  }
+  __device__ static uint32_t mul(uint32_t a, uint32_t b) {
+    const __half2 r = __hmul2(*reinterpret_cast<__half2*>(&a), *reinterpret_cast<__half2*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&r);
   }
 };
 
-template <typename T>
-__device__ __forceinline__ uint16_t small_int_bits(int n) {  // |n| <= 256, exact in bf16/fp16
-  const float f = __int_as_float(0x4B400000 + n) - 12582912.0f;  // exact for |n| < 2^22
-  if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-    return (uint16_t)(__float_as_uint(f) >> 16);  // <= 8 significant bits: truncation is exact
-  } else {
-    return __half_as_ushort(__float2half_rn(f));
-  }
+// |x| = m 2^(be - 1075) with m < 2^53, from the bits of a double or a float (a float's
+// significand shifted into a double's place); sgn: a word with x's sign in its top bit.
+// ANY: subnormals too; otherwise the leading one is taken for granted (a zero then has a
+// be that shifts it out).
+template <bool ANY>
+__device__ __forceinline__ void decode(double x, uint32_t& lo, uint32_t& hi, int& be, uint32_t& sgn) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  sgn = (uint32_t)(b >> 32);
+  lo = (uint32_t)b;
+  be = (int)((sgn >> 20) & 0x7FFu);
+  hi = (sgn & 0xFFFFFu) | (!ANY || be ? 0x100000u : 0u);
+  if constexpr (ANY) be = max(be, 1);
+}
+template <bool ANY>
+__device__ __forceinline__ void decode(float x, uint32_t& lo, uint32_t& hi, int& be, uint32_t& sgn) {
+  sgn = __float_as_uint(x);
+  be = (int)((sgn >> 23) & 0xFFu);
+  const uint32_t m = (sgn & 0x7FFFFFu) | (!ANY || be ? 0x800000u : 0u);
+  lo = m << 29;
+  hi = m >> 3;
+  if constexpr (ANY) be = max(be, 1);
+  be += 896;
 }
 
-template <typename T, int S, int t>
-__device__ __forceinline__ void slice_level(const SliceWindow (&w)[8], const bool (&neg)[8], uint32_t (&zp)[8],
-                                            uint8_t* base, int slice_stride, uint32_t soff) {
-  if constexpr (t <= S) {
-    uint16_t h[8];
-#pragma unroll
-    for (int u = 0; u < 8; u++) {
-      uint32_t zt = w[u].template z<kSplitBeta * (S - t)>();
-      if (neg[u]) zt = 0u - zt;
-      h[u] = small_int_bits<T>((int)(zt - (zp[u] << kSplitBeta)));
-      zp[u] = zt;
-    }
-    *reinterpret_cast<uint4*>(base + (size_t)(t - 1) * slice_stride + soff) = *reinterpret_cast<uint4*>(h);
-    slice_level<T, S, t + 1>(w, neg, zp, base, slice_stride, soff);
-  }
+// shifts that give 0 for a count beyond the width (a negative one counts as such)
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, int n) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+__device__ __forceinline__ unsigned long long shl64(unsigned long long v, int n) {
+  unsigned long long r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+__device__ __forceinline__ uint32_t shr32(uint32_t v, int n) {
+  uint32_t r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+  return r;
+}
+__device__ __forceinline__ uint32_t shl32(uint32_t v, int n) {
+  uint32_t r;
+  asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+  return r;
 }
 
-// x 2^-e = +-m 2^ex with an integer significand m, from the bits of a double or a float
-__device__ __forceinline__ void decode(double x, int e, bool& neg, unsigned long long& m, int& ex) {
-  const long long b = __double_as_longlong(x);
-  neg = b < 0;
-  const int be = (int)((b >> 52) & 0x7FF);
-  const unsigned long long frac = (unsigned long long)b & ((1ull << 52) - 1ull);
-  m = be ? (frac | (1ull << 52)) : frac;
-  ex = (be ? be : 1) - 1075 - e;
-}
-__device__ __forceinline__ void decode(float x, int e, bool& neg, unsigned long long& m, int& ex) {
-  const uint32_t b = __float_as_uint(x);
-  neg = (b >> 31) != 0;
-  const int be = (int)((b >> 23) & 0xFF);
-  const uint32_t frac = b & 0x7FFFFFu;
-  m = be ? (frac | 0x800000u) : frac;
-  ex = (be ? be : 1) - 150 - e;
+// V at an exact tie, moved off it to the side half-even rounds to (see above)
+template <int S, typename U>
+__device__ __forceinline__ U tie_to_even(U V) {
+  constexpr U kTies = (U)(2 * ((1ull << (7 * S)) - 1) / 127);  // bits p-1 of every level
+  const U low = V & ((U)0 - V) & kTies;
+  return low ? ((V & (low << 1)) ? V + 1 : V - 1) : V;
 }
 
-template <typename T, int S, typename E>
-__device__ __forceinline__ void slice_store8(const E (&x)[8], int e, uint8_t* base, int slice_stride, uint32_t soff) {
-  SliceWindow w[8];
-  bool neg[8];
-  uint32_t zp[8];
+// The window of one element, subnormals and tiny tiles included (r: the shift may be a left
+// one). Out of line: only tiles whose largest element is below 2^-900 need it.
+template <int S, typename E>
+__device__ __noinline__ unsigned long long slice_window_any(E x, int e) {
+  uint32_t lo, hi, sgn;
+  int be;
+  decode<true>(x, lo, hi, be, sgn);
+  const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+  const int sh = e + 1073 - 7 * S - be;  // V = m 2^-sh
+  if (sh < 1) return tie_to_even<S>(shl64(m, -sh));  // exact
+  const unsigned long long V = shr64(m, sh);
+  return sh < 64 && shl64(m, 64 - sh) == 0ull ? tie_to_even<S>(V) : V;
+}
+
+// The windows of 8 elements: V's low word, V >> 21, and the signs.
+template <int S, typename E>
+__device__ __forceinline__ void slice_windows(const E (&x)[8], int e, uint32_t (&w0)[8], uint32_t (&w1)[8],
+                                              uint32_t (&sgn)[8]) {
+  // A normal element of a tile with max|x| < 2^e has be <= e + 1022, so V = m >> sh with
+  // sh >= 51 - 7S. The significand's low kPre = 50 - 7S bits are below every V and with 4
+  // slices or fewer are dropped first: what is left fits 32 bits. A zero or subnormal
+  // element's be = 0 shifts everything out: V = 0, as it should be.
+  constexpr int kPre = 50 - 7 * S;
+  constexpr bool k32 = S <= 4;
+  const int c = e + 1073 - 7 * S;
+  uint32_t some = 0xFFFFFFFFu;  // 0: some element may have V even and no bit below it
 #pragma unroll
   for (int u = 0; u < 8; u++) {
-    unsigned long long m;
-    int ex;
-    decode(x[u], e, neg[u], m, ex);
-    w[u].init(m, -(ex + kSplitBeta * S));
-    zp[u] = 0u;
+    uint32_t lo, hi;
+    int be;
+    decode<false>(x[u], lo, hi, be, sgn[u]);
+    const int sh = c - be;
+    if constexpr (k32) {
+      const uint32_t m = kPre >= 32 ? hi >> (kPre & 31) : __funnelshift_r(lo, hi, kPre & 31);
+      const int r = sh - kPre;
+      w0[u] = shr32(m, r);
+      w1[u] = w0[u] >> 21;
+      // the dropped bits (a float's 24-bit significand has none below bit 29)
+      uint32_t cut = 0u;
+      if constexpr (kPre >= 32)
+        cut = lo | (hi & ((1u << (kPre & 31)) - 1u));
+      else if constexpr (!std::is_same<E, float>::value)
+        cut = lo & ((1u << (kPre & 31)) - 1u);
+      some = min(some, shl32(m, 31 - r) | cut);
+    } else {
+      const unsigned long long V = shr64(((unsigned long long)hi << 32) | lo, sh);
+      w0[u] = (uint32_t)V;
+      w1[u] = (uint32_t)(V >> 21);
+      some = min(some, shl32(lo, 31 - sh));
+    }
   }
-  slice_level<T, S, 1>(w, neg, zp, base, slice_stride, soff);
+  if (e <= -900) {
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      const unsigned long long V = slice_window_any<S>(x[u], e);
+      w0[u] = (uint32_t)V;
+      w1[u] = (uint32_t)(V >> 21);
+    }
+  } else if (some == 0u) {
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      uint32_t lo, hi, sg;
+      int be;
+      decode<false>(x[u], lo, hi, be, sg);
+      const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+      const int sh = c - be;
+      const bool exact = shl64(m, 64 - sh) == 0ull;  // no bit below V (V = 0 when sh is beyond m's width)
+      if constexpr (k32) {
+        w0[u] = exact ? tie_to_even<S>(w0[u]) : w0[u];
+        w1[u] = w0[u] >> 21;
+      } else if (exact) {
+        const unsigned long long V = tie_to_even<S>(shr64(m, sh));
+        w0[u] = (uint32_t)V;
+        w1[u] = (uint32_t)(V >> 21);
+      }
+    }
+  }
+}
+
+// Slice i levels above the finest (t = S - i): N_t as an exact float, without its sign.
+template <int S, int i>
+__device__ __forceinline__ float slice_digit(uint32_t w0, uint32_t w1) {
+  static_assert(S <= 6, "two windows of three levels");
+  constexpr int p = 2 + 7 * (i % 3);
+  constexpr uint32_t kMagic = 0x4B000000u;  // 2^23 as a float
+  const uint32_t w = i < 3 ? w0 : w1;
+  if constexpr (i == S - 1) {  // the top slice: N_1 = Z_1 <= 128
+    const uint32_t f = ((w + (1u << (p - 1))) & ~((1u << p) - 1u)) | kMagic;
+    return fmaf(__uint_as_float(f), 1.0f / (1 << p), -(float)(1 << (23 - p)));
+  } else {
+    const uint32_t r = (w & ((1u << p) - 1u)) ^ (1u << (p - 1));
+    const uint32_t ra = (w & ((1u << (p + 7)) - 1u)) ^ (1u << (p + 6));
+    const uint32_t f = ra - r + (kMagic + (1u << (p - 1)));
+    return fmaf(__uint_as_float(f), 1.0f / (1 << p), -(float)((1 << (23 - p)) + 64));
+  }
+}
+
+template <typename T, int S, int i>
+__device__ __forceinline__ void slice_levels(const uint32_t (&w0)[8], const uint32_t (&w1)[8],
+                                             const uint32_t (&sg)[4], uint8_t* dst, int slice_stride) {
+  if constexpr (i < S) {
+    uint32_t h[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++)
+      h[u] = Slice2<T>::mul(Slice2<T>::pack(slice_digit<S, i>(w0[2 * u], w1[2 * u]),
+                                            slice_digit<S, i>(w0[2 * u + 1], w1[2 * u + 1])),
+                            sg[u]);
+    *reinterpret_cast<uint4*>(dst + (size_t)(S - 1 - i) * slice_stride) = make_uint4(h[0], h[1], h[2], h[3]);
+    slice_levels<T, S, i + 1>(w0, w1, sg, dst, slice_stride);
+  }
+}
+
+// Slice 8 consecutive inner elements (one 16-byte chunk of a swizzled row) of one packed
+// row and store the S chunks.
+template <typename T, int S, typename E>
+__device__ __forceinline__ void slice_store8(const E (&x)[8], int e, uint8_t* dst, int slice_stride) {
+  uint32_t w0[8], w1[8], sgn[8], sg[4];
+  slice_windows<S>(x, e, w0, w1, sgn);
+#pragma unroll
+  for (int u = 0; u < 4; u++)
+    sg[u] = (__byte_perm(sgn[2 * u], sgn[2 * u + 1], 0x7632) & 0x80008000u) | Slice2<T>::kOnes;  // +-1 each
+  slice_levels<T, S, 0>(w0, w1, sg, dst, slice_stride);
 }
 
 // Complex elements (CPLX): the real product's A tile is [Ar, -Ai] (inner index kk' < q
@@ -496,131 +618,197 @@ __device__ __forceinline__ double neg_if(double v, bool n) {  // sign flip as bi
   return n ? __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull) : v;
 }
 
+// A CTA packs a group of 128 lines at one or several inner blocks: the rows of one A block,
+// or the columns of four B blocks that follow each other in the plan's list. It looks every
+// line up once (four dependent loads) and then makes passes of 256 pieces of 8 inner
+// elements: half a 32-deep chunk of the A block, or two chunks of a B block. A pass's loads
+// are in flight while the pass before is sliced. Groups are dealt to `ny` CTAs each, pass
+// by pass, when they are too few to fill the machine. Four neighbouring threads take one
+// line's 32 inner elements and a warp 8 lines, so every store instruction writes 512
+// contiguous bytes of the packed image, and loads read whole 32-byte sectors in either
+// storage order: 64 bytes of a line (in 16-byte loads where the line starts are aligned),
+// or 8 neighbouring lines' elements.
+constexpr int kPackThreads = 256;
+constexpr int kPackLines = 128;                             // lines of a group
+constexpr int kPackEntries = kPackLines / 32;               // B blocks of a group (32 columns each)
+constexpr int kPackMaxY = 8;
+constexpr int kPackResident = 3 * 152;                      // CTAs on the machine at once
+static_assert(kPackLines == kSplitBM, "an A group is one A block");
+
+// What a CTA looks up once per line ...
+struct PackLine {
+  int64_t base;   // the line's first element (real: E units; complex: doubles), -1: zeros
+  int32_t step;   // elements (doubles) from one inner index to the next
+  int32_t e;      // the line's exponent
+  int32_t cpart;  // complex B: 1 for the second half of the doubled columns
+};
+// ... and once per block
+struct PackEntry {
+  int64_t out;    // byte offset of the packed block
+  int32_t q, nkc; // inner elements, 32-deep chunks (0: no block)
+  int32_t pass0;  // its first pass
+};
+
 template <typename T, int S, typename E, bool CPLX = false>
-__global__ void __launch_bounds__(256) split_pack_kernel(SplitArgs a) {
-  constexpr int s = S;
-  const E* Ae = reinterpret_cast<const E*>(std::is_same<E, float>::value ? (const void*)a.Af : (const void*)a.A);
-  const E* Be = reinterpret_cast<const E*>(std::is_same<E, float>::value ? (const void*)a.Bf : (const void*)a.B);
-  if ((int)blockIdx.x < a.n_a_blocks) {
-    // A block (rb, kt): chunks of 128 rows x 32 inner elements
-    const int blk = a.a_blocks[blockIdx.x];
-    const int rb = blk / a.K, kt = blk % a.K;
-    const int q = a.q[kt];
-    const int nkc = (q + kSplitKC - 1) / kSplitKC;
-    uint8_t* out = a.apk + a.apk_off[blk];
-    for (int item = threadIdx.x; item < nkc * kSplitBM * 4; item += blockDim.x) {
-      const int ch = item & 3, rr = (item >> 2) % kSplitBM, kc = (item >> 2) / kSplitBM;
-      const int64_t m = (int64_t)rb * kSplitBM + rr;
-      E x[8];
-      int e = 0;
-      bool present = false;
-      int64_t off = -1;
-      int i = 0;
-      if (m < a.Mtot) {
-        i = a.row_tile[m];
-        present = a.am[(int64_t)i * a.K + kt] != 0;
-        off = a.transa ? a.a_off[(int64_t)kt * a.M + i] : a.a_off[(int64_t)i * a.K + kt];
-        if (present && off < 0) {
-          atomicOr(a.err, kErrBadOffset);
-          present = false;
+__global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __grid_constant__ SplitArgs a, int ny) {
+  __shared__ PackLine lines[kPackLines];
+  __shared__ PackEntry entries[kPackEntries];
+  __shared__ int passes_of[kPackEntries];
+  constexpr int VE = 16 / (int)sizeof(E);
+  const int tid = threadIdx.x;
+  const int grp = blockIdx.x / ny;
+  const bool isA = grp < a.n_a_blocks;
+  const bool contig = isA ? !a.transa : a.transb != 0;  // a line's inner elements are contiguous
+  if (tid < kPackLines) {
+    const int en = isA ? 0 : tid >> 5, ln = isA ? tid : tid & 31;
+    const int at = isA ? grp : (grp - a.n_a_blocks) * kPackEntries + en;
+    PackLine l{-1, 1, 0, 0};
+    PackEntry pe{0, 0, 0, 0};
+    if (isA || at < a.n_b_blocks) {
+      const int blk = isA ? a.a_blocks[at] : a.b_blocks[at];
+      const int kt = isA ? blk % a.K : blk / a.CB;
+      const int64_t x = (isA ? (int64_t)(blk / a.K) * kSplitBM : (int64_t)(blk % a.CB) * 32) + ln;
+      const int q = a.q[kt];
+      pe.out = isA ? a.apk_off[blk] : a.bpk_off[blk];
+      pe.q = q;
+      pe.nkc = (q + kSplitKC - 1) / kSplitKC;
+      if (x < (isA ? a.Mtot : a.Ntot)) {
+        const int t = isA ? a.row_tile[x] : a.col_tile[x];
+        const int64_t tile = isA ? (int64_t)t * a.K + kt : (int64_t)kt * a.N + t;
+        const int64_t off = isA ? (a.transa ? a.a_off[(int64_t)kt * a.M + t] : a.a_off[tile])
+                                : (a.transb ? a.b_off[(int64_t)t * a.K + kt] : a.b_off[tile]);
+        const int width = isA ? a.r[t] : a.c[t];  // lines of the tile
+        int64_t lx = x - (isA ? a.ro[t] : a.co[t]);
+        if (!isA && CPLX && lx >= (width >> 1)) {
+          l.cpart = 1;
+          lx -= width >> 1;
         }
-        e = a.rowscale ? a.eArow[(int64_t)kt * a.Mtot + m] : a.eA[(int64_t)i * a.K + kt];
-      }
-      const int64_t lr = m - (m < a.Mtot ? a.ro[i] : 0);
-      // element (lr, k) of A_ik at line + k * step, stored transposed or not
-      const int64_t step = a.transa ? (m < a.Mtot ? a.r[i] : 0) : 1;
-      const int k0 = kc * kSplitKC + ch * 8;
-      if constexpr (CPLX) {
-        // complex element (lr, kc) of the tile at row + 2 kc cstep (cstep = 1, or the tile's
-        // row count when stored transposed); part 0 real, 1 imaginary
-        const int qc = q >> 1;
-        const int64_t cstep = a.transa ? step : 1;
-        const double* row = a.A + 2 * (off + (a.transa ? lr : lr * qc));
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-          const int kk = k0 + u, part = kk >= qc;
-          x[u] = (present && kk < q) ? neg_if(__ldg(row + 2 * (kk - part * qc) * cstep + part), part) : 0.0;
+        if (isA ? a.am[tile] : a.bm[tile]) {
+          // (an offset off the 16-byte grid is reported, never read with 16-byte loads)
+          if (off < 0 || (!CPLX && contig && q % VE == 0 && off % VE != 0)) {
+            atomicOr(a.err, kErrBadOffset);
+          } else if (CPLX) {
+            const int64_t tw = isA ? width : width >> 1;
+            l.base = 2 * (off + (contig ? lx * (q >> 1) : lx));
+            l.step = contig ? 2 : (int)(2 * tw);
+          } else {
+            l.base = off + (contig ? lx * q : lx);
+            l.step = contig ? 1 : width;
+          }
         }
-      } else {
-        const E* line = Ae + off + (a.transa ? lr : lr * q);
-#pragma unroll
-        for (int u = 0; u < 8; u++) x[u] = (present && k0 + u < q) ? __ldg(line + (k0 + u) * step) : E(0);
+        l.e = a.rowscale ? (isA ? a.eArow[(int64_t)kt * a.Mtot + x] : a.eBcol[(int64_t)kt * a.Ntot + x])
+                         : (isA ? a.eA[tile] : a.eB[tile]);
       }
-      slice_store8<T, S>(x, e, out + (size_t)kc * s * kAChunk, kAChunk, swz64(rr, ch * 8));
     }
-  } else {
-    // B block (kt, cb): chunks of tn rows (columns of B) x 32 inner elements, transposed
-    const int blk = a.b_blocks[blockIdx.x - a.n_a_blocks];
-    const int kt = blk / a.CB, cb = blk % a.CB;
-    const int q = a.q[kt];
-    const int tn = a.tn;
-    const int nkc = (q + kSplitKC - 1) / kSplitKC;
-    const int bchunk = tn * kSplitKC * 2;
-    uint8_t* out = a.bpk + a.bpk_off[blk];
-    for (int item = threadIdx.x; item < nkc * tn * 4; item += blockDim.x) {
-      const int nn = item % tn, ch = (item / tn) & 3, kc = (item / tn) >> 2;
-      const int64_t n = (int64_t)cb * tn + nn;
-      E x[8];
-      int e = 0;
-      bool present = false;
-      int64_t off = -1;
-      int j = 0, cj = 0;
-      if (n < a.Ntot) {
-        j = a.col_tile[n];
-        cj = a.c[j];
-        present = a.bm[(int64_t)kt * a.N + j] != 0;
-        off = a.transb ? a.b_off[(int64_t)j * a.K + kt] : a.b_off[(int64_t)kt * a.N + j];
-        if (present && off < 0) {
-          atomicOr(a.err, kErrBadOffset);
-          present = false;
-        }
-        e = a.rowscale ? a.eBcol[(int64_t)kt * a.Ntot + n] : a.eB[(int64_t)kt * a.N + j];
-      }
-      const int64_t lc = n - (n < a.Ntot ? a.co[j] : 0);
-      // element (k, lc) of B_kj at line + k * step, stored transposed or not
-      const int64_t step = a.transb ? 1 : cj;
-      const int k0 = kc * kSplitKC + ch * 8;
-      if constexpr (CPLX) {
-        // complex element (kc, c) of the tile at col + 2 kc kstep: kstep = the tile's complex
-        // column count, or 1 when stored transposed (then column c starts c * qc in)
-        const int qc = q >> 1, cc = cj >> 1;
-        const int cpart = lc >= cc;
-        const int64_t kstep = a.transb ? 1 : cc;
-        const double* col = a.B + 2 * (off + (lc - cpart * cc) * (a.transb ? qc : 1));
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-          const int kk = k0 + u, rpart = kk >= qc;
-          x[u] = (present && kk < q)
-                     ? neg_if(__ldg(col + 2 * (int64_t)(kk - rpart * qc) * kstep + (rpart ^ cpart)), rpart & cpart)
-                     : 0.0;
-        }
-      } else {
-        const E* line = Be + off + (a.transb ? lc * q : lc);
-#pragma unroll
-        for (int u = 0; u < 8; u++) x[u] = (present && k0 + u < q) ? __ldg(line + (k0 + u) * step) : E(0);
-      }
-      slice_store8<T, S>(x, e, out + (size_t)kc * s * bchunk, bchunk, swz64(nn, ch * 8));
+    lines[tid] = l;
+    if (ln == 0) {
+      entries[en] = pe;
+      passes_of[en] = isA ? 2 * pe.nkc : (pe.nkc + 1) >> 1;
     }
+  }
+  __syncthreads();
+  int total = 0;
+  for (int en = 0; en < (isA ? 1 : kPackEntries); en++) total += passes_of[en];
+
+  const E* const src = isA ? reinterpret_cast<const E*>(std::is_same<E, float>::value ? (const void*)a.Af : (const void*)a.A)
+                           : reinterpret_cast<const E*>(std::is_same<E, float>::value ? (const void*)a.Bf : (const void*)a.B);
+  const int slice_stride = isA ? kSplitBM * kSplitKC * 2 : 32 * kSplitKC * 2;
+  uint8_t* const pk = isA ? a.apk : a.bpk;
+  const int ch = tid & 3;
+
+  struct Piece {  // a thread's 8 elements of a pass
+    E x[8];
+    int line;  // -1: none
+    int k0;    // first inner index, or past the end: zeros
+    uint8_t* dst;
+  };
+  auto load = [&](Piece& pc, int pass) {
+    int en = 0, p = pass;
+    while (p >= passes_of[en]) p -= passes_of[en++];
+    const PackEntry pe = entries[en];
+    // A: pass p is half p & 1 of chunk p >> 1; B: chunks 2p and 2p + 1
+    const int ln = isA ? (p & 1) * 64 + (tid >> 2) : (tid >> 2) & 31;
+    const int kc = isA ? p >> 1 : 2 * p + (tid >> 7);
+    pc.line = kc < pe.nkc ? (isA ? ln : en * 32 + ln) : -1;
+    pc.dst = pk + pe.out + (size_t)kc * S * slice_stride + swz64(ln, ch * 8);
+    const int q = pe.q;
+    int k0 = kc * kSplitKC + ch * 8;
+    const PackLine l = lines[isA ? ln : en * 32 + ln];
+    if (l.base < 0) k0 = 1 << 30;
+    pc.k0 = k0 < q ? k0 : 1 << 30;
+    if constexpr (CPLX) {
+      // inner index kk takes part (kk >= q/2) of the complex inner index; its sign and part
+      // follow the block form above
+      const int qc = q >> 1;
+#pragma unroll
+      for (int u = 0; u < 8; u++) {
+        const int kk = k0 + u, part = kk >= qc;
+        const bool neg = isA ? part : (part & l.cpart);
+        pc.x[u] = kk < q ? neg_if(__ldg(src + l.base + (int64_t)(kk - part * qc) * l.step + (part ^ l.cpart)), neg) : 0.0;
+      }
+    } else if (contig && q % VE == 0) {
+      // lines of whole 16-byte vectors (tiles start on 16 bytes)
+      const uint4* const v4 = reinterpret_cast<const uint4*>(src + l.base + k0);
+#pragma unroll
+      for (int v = 0; v < 8 / VE; v++) {
+        uint4 r = make_uint4(0u, 0u, 0u, 0u);
+        if (k0 + v * VE < q) r = __ldg(v4 + v);
+        *reinterpret_cast<uint4*>(&pc.x[v * VE]) = r;
+      }
+    } else {
+      const E* const v = src + l.base + (int64_t)k0 * l.step;
+      const int64_t step = l.step;
+#pragma unroll
+      for (int u = 0; u < 8; u++) pc.x[u] = k0 + u < q ? __ldg(v + u * step) : E(0);
+    }
+  };
+  auto store = [&](const Piece& pc) {
+    if (pc.line < 0) return;
+    if (pc.k0 < 1 << 30) {
+      slice_store8<T, S>(pc.x, lines[pc.line].e, pc.dst, slice_stride);
+    } else {  // an absent tile's line, or past the inner block's end
+#pragma unroll
+      for (int t = 0; t < S; t++)
+        *reinterpret_cast<uint4*>(pc.dst + (size_t)t * slice_stride) = make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  int pass = blockIdx.x % ny;
+  if (pass >= total) return;
+  Piece cur, nxt;
+  load(cur, pass);
+  for (;;) {
+    pass += ny;
+    const bool more = pass < total;
+    if (more) load(nxt, pass);
+    store(cur);
+    if (!more) break;
+    cur = nxt;
   }
 }
 
 }  // namespace
 
 template <typename E, bool C = false>
-cudaError_t launch_pack(const SplitArgs& a, unsigned g, cudaStream_t st) {
+cudaError_t launch_pack(const SplitArgs& a, cudaStream_t st) {
+  // CTAs per group: one, or as many (up to a pass each) as fill the resident grid, where a
+  // group's passes one after the other would be most of a small product's time
+  const int groups = a.n_a_blocks + (a.n_b_blocks + kPackEntries - 1) / kPackEntries;
+  const int passes = 2 * ((a.qmax + kSplitKC - 1) / kSplitKC);
+  const int ny = std::max(1, std::min({kPackMaxY, passes, kPackResident / std::max(1, groups)}));
+  const unsigned g = (unsigned)(groups * ny);
   switch (a.s * 2 + (a.fp16 ? 1 : 0)) {
-    case 2: split_pack_kernel<__nv_bfloat16, 1, E, C><<<g, 256, 0, st>>>(a); break;
-    case 3: split_pack_kernel<__half, 1, E, C><<<g, 256, 0, st>>>(a); break;
-    case 4: split_pack_kernel<__nv_bfloat16, 2, E, C><<<g, 256, 0, st>>>(a); break;
-    case 5: split_pack_kernel<__half, 2, E, C><<<g, 256, 0, st>>>(a); break;
-    case 6: split_pack_kernel<__nv_bfloat16, 3, E, C><<<g, 256, 0, st>>>(a); break;
-    case 7: split_pack_kernel<__half, 3, E, C><<<g, 256, 0, st>>>(a); break;
-    case 8: split_pack_kernel<__nv_bfloat16, 4, E, C><<<g, 256, 0, st>>>(a); break;
-    case 9: split_pack_kernel<__half, 4, E, C><<<g, 256, 0, st>>>(a); break;
-    case 10: split_pack_kernel<__nv_bfloat16, 5, E, C><<<g, 256, 0, st>>>(a); break;
-    case 11: split_pack_kernel<__half, 5, E, C><<<g, 256, 0, st>>>(a); break;
-    case 12: split_pack_kernel<__nv_bfloat16, 6, E, C><<<g, 256, 0, st>>>(a); break;
-    case 13: split_pack_kernel<__half, 6, E, C><<<g, 256, 0, st>>>(a); break;
+    case 2: split_pack_kernel<__nv_bfloat16, 1, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 3: split_pack_kernel<__half, 1, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 4: split_pack_kernel<__nv_bfloat16, 2, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 5: split_pack_kernel<__half, 2, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 6: split_pack_kernel<__nv_bfloat16, 3, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 7: split_pack_kernel<__half, 3, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 8: split_pack_kernel<__nv_bfloat16, 4, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 9: split_pack_kernel<__half, 4, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 10: split_pack_kernel<__nv_bfloat16, 5, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 11: split_pack_kernel<__half, 5, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 12: split_pack_kernel<__nv_bfloat16, 6, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 13: split_pack_kernel<__half, 6, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -655,9 +843,7 @@ cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* 
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (a.n_a_blocks + a.n_b_blocks > 0) {
-    const unsigned g = (unsigned)(a.n_a_blocks + a.n_b_blocks);
-    cudaError_t pe = a.f32 ? launch_pack<float>(a, g, st)
-                           : a.cplx ? launch_pack<double, true>(a, g, st) : launch_pack<double>(a, g, st);
+    cudaError_t pe = a.f32 ? launch_pack<float>(a, st) : a.cplx ? launch_pack<double, true>(a, st) : launch_pack<double>(a, st);
     if (pe != cudaSuccess) return pe;
   }
   if (ev) cudaEventRecord(ev[++*k], st);
