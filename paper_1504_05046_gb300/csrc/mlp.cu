@@ -13,8 +13,10 @@
 // and deviations, two tanh layers, one linear output = standardised log time.
 // Parameters in one float vector: W1[H][F], b1[H], W2[H][H], b2[H], w3[H], b3.
 // Training: full-batch mean squared error, Adam; every reduction over samples runs in
-// a fixed order (per-block partial sums, then a sum over blocks in block order), so
-// training is bit-for-bit reproducible.
+// a fixed order (partial sums over tiles of 128 samples, then a sum over the tiles in tile
+// order), so training is bit-for-bit reproducible.
+#include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -30,7 +32,7 @@ constexpr int F = BSMM_NFEATURES;
 constexpr int H = 32;
 constexpr int NP = H * F + H + H * H + H + H + 1;
 constexpr int OW1 = 0, OB1 = H * F, OW2 = OB1 + H, OB2 = OW2 + H * H, OW3 = OB2 + H, OB3 = OW3 + H;
-constexpr int TILE = 128;  // samples per block in the gradient kernel
+constexpr int TILE = 128;  // samples per partial sum of the gradient
 
 struct Norm {
   float xmu[F], xsd[F];
@@ -71,98 +73,338 @@ __global__ void mlp_predict_kernel(const float* __restrict__ params, Norm nm, co
   y[s] = o * nm.ysd + nm.ymu;  // log time in the caller's units
 }
 
-// Per block: the loss and gradient contributions of its TILE samples, summed in
-// sample order, written to part[block][0..NP] (entry NP = sum of squared residuals).
-__global__ void __launch_bounds__(TILE) mlp_grad_kernel(const float* __restrict__ params, Norm nm,
-                                                        const float* __restrict__ X, const float* __restrict__ t,
-                                                        int64_t n, float* __restrict__ part) {
-  extern __shared__ float sm[];
-  float* w = sm;                 // NP
-  float* xs = w + NP;            // TILE x F
-  float* h1s = xs + TILE * F;    // TILE x H
-  float* h2s = h1s + TILE * H;   // TILE x H
-  float* d1s = h2s + TILE * H;   // TILE x H  (dL/dz1)
-  float* d2s = d1s + TILE * H;   // TILE x H  (dL/dz2)
-  float* dys = d2s + TILE * H;   // TILE      (dL/dy)
-  float* r2s = dys + TILE;       // TILE      squared residuals
-  for (int p = threadIdx.x; p < NP; p += blockDim.x) w[p] = params[p];
+// Training: one cooperative launch for every step of a fit. Per step, CTAs take tiles of
+// TILE samples (forward, backward, the tile's gradient sums in sample order, written to
+// part[tile][0..NP], entry NP the sum of squared residuals); after a grid barrier each CTA
+// adds a few parameters' partial sums in tile order and applies Adam; after a second barrier
+// the next step reads the new parameters.
+// A step is a chain of latencies (20000 samples are 12 MFLOP per layer pass), so the layout
+// serves those and the shared-memory port, which all 16 warps share: a warp takes 8 samples
+// through the whole network, lane = neuron, the neuron's weights in registers and the
+// samples' activations read by broadcast, so no barrier is needed before the gradient sums;
+// those take 2 x 4 parameters per thread; a parameter's partial sums are fetched by the
+// whole CTA at once, and its Adam state stays in its thread. Every sum keeps one order.
+// 20000 samples: 22 us per step (the network and its sums 7.5 us per tile, which is what
+// their shared-memory reads take; 157 tiles on 152 SMs; a barrier 2 us). As three launches
+// per step, with a thread per sample striding through its own rows of shared memory (32-way
+// conflicts) and 128 threads for the 1506 gradient sums: 95 us.
+constexpr int kTrainThreads = 512;
+constexpr int kWarpSamples = TILE / (kTrainThreads / 32);  // 8
+constexpr int LD = H + 4;        // row of neurons, padded: 8 rows cover the banks
+constexpr int kGather = 4096;    // partial sums fetched at a time
+constexpr int kKeep = 2;         // tiles of a CTA whose standardised inputs stay in shared memory
+constexpr int64_t kBarrierNs = 4000000000LL;  // bounded wait at a grid barrier
+constexpr int kNPpad = (NP + 3) / 4 * 4;      // parameter arrays hold whole 16-byte vectors
+
+struct TrainShared {
+  float w1[kNPpad];              // every parameter, as in global memory ...
+  float w2[H][LD];               // ... and W2 again in padded rows
+  float xs[kKeep][TILE][F];
+  float ts[kKeep][TILE];
+  float h1[TILE][LD], h2[TILE][LD], d1[TILE][LD], d2[TILE][LD];
+  float dy[TILE], r2[TILE];
+  float gather[kGather];
+};
+
+__device__ __forceinline__ int64_t now_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return (int64_t)t;
+}
+
+// Every CTA of the (cooperative) grid arrives; false when the wait ran out. `count` only
+// grows, by gridDim.x per barrier; sync[1] is the error flag.
+__device__ bool grid_barrier(unsigned* sync, unsigned target) {
   __syncthreads();
-  const int tid = threadIdx.x;
-  const int64_t s = (int64_t)blockIdx.x * TILE + tid;
-  float* x = xs + tid * F;
-  float* h1 = h1s + tid * H;
-  float* h2 = h2s + tid * H;
-  float* d1 = d1s + tid * H;
-  float* d2 = d2s + tid * H;
-  if (s < n) {
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&sync[0], 1u);
+    const int64_t t0 = now_ns();
+    unsigned spin = 0;
+    while ((int)(*(volatile unsigned*)&sync[0] - target) < 0) {  // (the count may wrap)
+      if (*(volatile unsigned*)&sync[1]) break;
+      if ((++spin & 1023u) == 0 && now_ns() - t0 > kBarrierNs) {
+        atomicExch(&sync[1], 1u);
+        break;
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return *(volatile unsigned*)&sync[1] == 0u;
+}
+
+// Sums over the tile's samples, in sample order: g[j][i] = sum a[q][j0 + j] b[q][i0 + i]
+template <int LDB>
+__device__ __forceinline__ void outer_sums(const float (*a)[LD], int j0, const float (*b)[LDB], int i0,
+                                           float (&g)[2][4]) {
 #pragma unroll
-    for (int f = 0; f < F; f++) x[f] = (X[s * F + f] - nm.xmu[f]) / nm.xsd[f];
-    float y;
-    mlp_forward_one(w, x, h1, h2, y);
-    const float r = y - (t[s] - nm.ymu) / nm.ysd;
-    const float dy = 2.0f * r / (float)n;
-    dys[tid] = dy;
-    r2s[tid] = r * r;
-    for (int j = 0; j < H; j++) d2[j] = dy * w[OW3 + j] * (1.0f - h2[j] * h2[j]);
-    for (int i = 0; i < H; i++) {
-      float g = 0.0f;
-      for (int j = 0; j < H; j++) g = fmaf(w[OW2 + j * H + i], d2[j], g);
-      d1[i] = g * (1.0f - h1[i] * h1[i]);
+  for (int j = 0; j < 2; j++)
+#pragma unroll
+    for (int i = 0; i < 4; i++) g[j][i] = 0.0f;
+#pragma unroll 4
+  for (int q = 0; q < TILE; q++) {
+    const float2 av = *reinterpret_cast<const float2*>(&a[q][j0]);
+    const float4 bv = *reinterpret_cast<const float4*>(&b[q][i0]);
+    g[0][0] = fmaf(av.x, bv.x, g[0][0]);
+    g[0][1] = fmaf(av.x, bv.y, g[0][1]);
+    g[0][2] = fmaf(av.x, bv.z, g[0][2]);
+    g[0][3] = fmaf(av.x, bv.w, g[0][3]);
+    g[1][0] = fmaf(av.y, bv.x, g[1][0]);
+    g[1][1] = fmaf(av.y, bv.y, g[1][1]);
+    g[1][2] = fmaf(av.y, bv.z, g[1][2]);
+    g[1][3] = fmaf(av.y, bv.w, g[1][3]);
+  }
+}
+__device__ __forceinline__ float column_sum(const float (*a)[LD], int j) {
+  float g = 0.0f;
+#pragma unroll 16
+  for (int q = 0; q < TILE; q++) g += a[q][j];
+  return g;
+}
+__device__ __forceinline__ float vector_sum(const float* a) {
+  float g = 0.0f;
+#pragma unroll 4
+  for (int q = 0; q < TILE; q += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(a + q);
+    g += v.x;
+    g += v.y;
+    g += v.z;
+    g += v.w;
+  }
+  return g;
+}
+
+// One tile's partial sums: out[0..NP]; slot: where its inputs are (or go)
+__device__ void train_tile(TrainShared& sm, const Norm& nm, const float* __restrict__ X, const float* __restrict__ t,
+                           int64_t n, int tile, int slot, bool kept, float* __restrict__ out) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int q0 = warp * kWarpSamples;  // this warp's samples
+  const int64_t s0 = (int64_t)tile * TILE;
+  float(*const xs)[F] = sm.xs[slot];
+  float* const ts = sm.ts[slot];
+  if (!kept) {  // standardised inputs and targets of the warp's samples
+    for (int e = lane; e < kWarpSamples * F; e += 32) {
+      const int f = e % F, q = q0 + e / F;
+      xs[q][f] = s0 + q < n ? (X[(s0 + q) * F + f] - nm.xmu[f]) / nm.xsd[f] : 0.0f;
     }
-  } else {
-    for (int f = 0; f < F; f++) x[f] = 0.0f;
-    for (int j = 0; j < H; j++) h1[j] = h2[j] = d1[j] = d2[j] = 0.0f;
-    dys[tid] = 0.0f;
-    r2s[tid] = 0.0f;
+    if (lane < kWarpSamples) ts[q0 + lane] = s0 + q0 + lane < n ? (t[s0 + q0 + lane] - nm.ymu) / nm.ysd : 0.0f;
+    __syncwarp();
+  }
+  const float* const w = sm.w1;
+  float h1[kWarpSamples], h2[kWarpSamples];
+  {
+    float wr[F], z[kWarpSamples];
+#pragma unroll
+    for (int f = 0; f < F; f += 4) *reinterpret_cast<float4*>(wr + f) = *reinterpret_cast<const float4*>(w + OW1 + lane * F + f);
+#pragma unroll
+    for (int u = 0; u < kWarpSamples; u++) z[u] = w[OB1 + lane];
+#pragma unroll
+    for (int f = 0; f < F; f += 4)
+#pragma unroll
+      for (int u = 0; u < kWarpSamples; u++) {
+        const float4 x = *reinterpret_cast<const float4*>(&xs[q0 + u][f]);
+        z[u] = fmaf(wr[f], x.x, z[u]);
+        z[u] = fmaf(wr[f + 1], x.y, z[u]);
+        z[u] = fmaf(wr[f + 2], x.z, z[u]);
+        z[u] = fmaf(wr[f + 3], x.w, z[u]);
+      }
+#pragma unroll
+    for (int u = 0; u < kWarpSamples; u++) {
+      h1[u] = s0 + q0 + u < n ? tanhf(z[u]) : 0.0f;
+      sm.h1[q0 + u][lane] = h1[u];
+    }
+  }
+  __syncwarp();
+  {
+    float z[kWarpSamples];
+#pragma unroll
+    for (int u = 0; u < kWarpSamples; u++) z[u] = w[OB2 + lane];
+#pragma unroll
+    for (int i = 0; i < H; i += 4) {
+      const float4 wr = *reinterpret_cast<const float4*>(&sm.w2[lane][i]);
+#pragma unroll
+      for (int u = 0; u < kWarpSamples; u++) {
+        const float4 h = *reinterpret_cast<const float4*>(&sm.h1[q0 + u][i]);
+        z[u] = fmaf(wr.x, h.x, z[u]);
+        z[u] = fmaf(wr.y, h.y, z[u]);
+        z[u] = fmaf(wr.z, h.z, z[u]);
+        z[u] = fmaf(wr.w, h.w, z[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kWarpSamples; u++) {
+      h2[u] = s0 + q0 + u < n ? tanhf(z[u]) : 0.0f;
+      sm.h2[q0 + u][lane] = h2[u];
+    }
+  }
+  __syncwarp();
+  float dy = 0.0f;
+  if (lane < kWarpSamples) {  // lane = sample: the output and its residual
+    const int q = q0 + lane;
+    float o = w[OB3];
+#pragma unroll
+    for (int i = 0; i < H; i += 4) {
+      const float4 h = *reinterpret_cast<const float4*>(&sm.h2[q][i]);
+      o = fmaf(w[OW3 + i], h.x, o);
+      o = fmaf(w[OW3 + i + 1], h.y, o);
+      o = fmaf(w[OW3 + i + 2], h.z, o);
+      o = fmaf(w[OW3 + i + 3], h.w, o);
+    }
+    const float r = o - ts[q];
+    const bool in = s0 + q < n;
+    dy = in ? 2.0f * r / (float)n : 0.0f;
+    sm.dy[q] = dy;
+    sm.r2[q] = in ? r * r : 0.0f;
+  }
+  {
+    const float w3 = w[OW3 + lane];
+#pragma unroll
+    for (int u = 0; u < kWarpSamples; u++) {
+      const float d = __shfl_sync(0xffffffffu, dy, u);
+      sm.d2[q0 + u][lane] = s0 + q0 + u < n ? d * w3 * (1.0f - h2[u] * h2[u]) : 0.0f;
+    }
+  }
+  __syncwarp();
+  {
+    float g[kWarpSamples];
+#pragma unroll
+    for (int u = 0; u < kWarpSamples; u++) g[u] = 0.0f;
+#pragma unroll
+    for (int j = 0; j < H; j += 4) {
+      const float wa = sm.w2[j][lane], wb = sm.w2[j + 1][lane], wc = sm.w2[j + 2][lane], wd = sm.w2[j + 3][lane];
+#pragma unroll
+      for (int u = 0; u < kWarpSamples; u++) {
+        const float4 d = *reinterpret_cast<const float4*>(&sm.d2[q0 + u][j]);
+        g[u] = fmaf(wa, d.x, g[u]);
+        g[u] = fmaf(wb, d.y, g[u]);
+        g[u] = fmaf(wc, d.z, g[u]);
+        g[u] = fmaf(wd, d.w, g[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kWarpSamples; u++)
+      sm.d1[q0 + u][lane] = s0 + q0 + u < n ? g[u] * (1.0f - h1[u] * h1[u]) : 0.0f;
   }
   __syncthreads();
-  float* out = part + (int64_t)blockIdx.x * (NP + 1);
-  for (int p = tid; p <= NP; p += blockDim.x) {
-    float g = 0.0f;
-    if (p < OB1) {
-      const int j = p / F, f = p % F;
-      for (int q = 0; q < TILE; q++) g = fmaf(d1s[q * H + j], xs[q * F + f], g);
-    } else if (p < OW2) {
-      const int j = p - OB1;
-      for (int q = 0; q < TILE; q++) g += d1s[q * H + j];
-    } else if (p < OB2) {
-      const int j = (p - OW2) / H, i = (p - OW2) % H;
-      for (int q = 0; q < TILE; q++) g = fmaf(d2s[q * H + j], h1s[q * H + i], g);
-    } else if (p < OW3) {
-      const int j = p - OB2;
-      for (int q = 0; q < TILE; q++) g += d2s[q * H + j];
-    } else if (p < OB3) {
-      const int i = p - OW3;
-      for (int q = 0; q < TILE; q++) g = fmaf(dys[q], h2s[q * H + i], g);
-    } else if (p == OB3) {
-      for (int q = 0; q < TILE; q++) g += dys[q];
-    } else {  // p == NP: loss numerator
-      for (int q = 0; q < TILE; q++) g += r2s[q];
+  // gradient sums over the tile's samples: warps 0-3 W2, 4-5 W1, 6-8 the single rows, 9 the rest
+  if (warp < 4) {
+    const int j = 2 * (warp * 4 + (lane >> 3)), i = 4 * (lane & 7);
+    float g[2][4];
+    outer_sums(sm.d2, j, sm.h1, i, g);
+#pragma unroll
+    for (int u = 0; u < 8; u++) out[OW2 + (j + u / 4) * H + i + u % 4] = g[u / 4][u % 4];
+  } else if (warp < 6) {
+    const int e = tid - 128;
+    if (e < 48) {
+      const int j = 2 * (e / 3), f = 4 * (e % 3);
+      float g[2][4];
+      outer_sums(sm.d1, j, xs, f, g);
+#pragma unroll
+      for (int u = 0; u < 8; u++) out[OW1 + (j + u / 4) * F + f + u % 4] = g[u / 4][u % 4];
     }
-    out[p] = g;
+  } else if (warp == 6) {
+    out[OB1 + lane] = column_sum(sm.d1, lane);
+  } else if (warp == 7) {
+    out[OB2 + lane] = column_sum(sm.d2, lane);
+  } else if (warp == 8) {
+    float g = 0.0f;
+#pragma unroll 16
+    for (int q = 0; q < TILE; q++) g = fmaf(sm.dy[q], sm.h2[q][lane], g);
+    out[OW3 + lane] = g;
+  } else if (warp == 9) {
+    if (lane < 2) out[OB3 + lane] = vector_sum(lane ? sm.r2 : sm.dy);  // OB3, then NP: the residuals
   }
+  __syncthreads();
 }
+static_assert(OB3 + 1 == NP, "the residual sum follows the last parameter");
 
-// grad[p] = sum over blocks in block order; grad[NP] = mean squared residual
-__global__ void mlp_reduce_kernel(const float* __restrict__ part, int nblocks, int64_t n, float* __restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > NP) return;
-  float g = 0.0f;
-  for (int b = 0; b < nblocks; b++) g += part[(int64_t)b * (NP + 1) + p];
-  grad[p] = p == NP ? g / (float)n : g;
-}
-
-__global__ void mlp_adam_kernel(float* __restrict__ params, float* __restrict__ m, float* __restrict__ v,
-                                const float* __restrict__ grad, float lr, float c1, float c2) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= NP) return;
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float g = grad[p];
-  const float mm = b1 * m[p] + (1.0f - b1) * g;
-  const float vv = b2 * v[p] + (1.0f - b2) * g * g;
-  m[p] = mm;
-  v[p] = vv;
-  params[p] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+// `total` passes over the samples; the first `updates` of them end in an Adam step, the
+// others leave the gradient (and grad[NP] = the mean squared residual) in grad.
+__global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(float* params, float* m, float* v, float* grad,
+                                                                  float* part, const __grid_constant__ Norm nm,
+                                                                  const float* __restrict__ X,
+                                                                  const float* __restrict__ t, int64_t n, int tiles,
+                                                                  int total, int updates, float lr, unsigned* sync) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  TrainShared& sm = *reinterpret_cast<TrainShared*>(raw);
+  const int tid = threadIdx.x, G = gridDim.x;
+  const int per = (NP + 1 + G - 1) / G;  // parameters whose sums this CTA adds
+  const int p0 = blockIdx.x * per, np = max(0, min(per, NP + 1 - p0));
+  double b1k = 1.0, b2k = 1.0;
+  float mp = 0.0f, vp = 0.0f, pp = 0.0f;  // the parameter and Adam state of a thread that owns one
+  const bool own = np <= kTrainThreads;
+  if (own && tid < np && p0 + tid < NP) {
+    mp = m[p0 + tid];
+    vp = v[p0 + tid];
+    pp = params[p0 + tid];
+  }
+  for (int it = 0; it < total; it++) {
+    if (tid < kNPpad / 4) {
+      const float4 w4 = __ldcg(reinterpret_cast<const float4*>(params) + tid);
+      reinterpret_cast<float4*>(sm.w1)[tid] = w4;
+      const int e = 4 * tid - OW2;  // (OW2 and H are multiples of 4)
+      if (e >= 0 && e < H * H) *reinterpret_cast<float4*>(&sm.w2[e / H][e % H]) = w4;
+    }
+    __syncthreads();
+    const bool keep = tiles <= kKeep * G;
+    for (int tile = blockIdx.x, k = 0; tile < tiles; tile += G, k++)
+      train_tile(sm, nm, X, t, n, tile, keep ? k : 0, keep && it > 0, part + (int64_t)tile * (NP + 1));
+    if (!grid_barrier(sync, (unsigned)(2 * it + 1) * G)) return;
+    // sums over the tiles in tile order: the CTA fetches a batch of its parameters' partial
+    // sums at once, then a thread per parameter adds them
+    const bool update = it < updates;
+    if (update) {
+      b1k = __dmul_rn(b1k, 0.9);
+      b2k = __dmul_rn(b2k, 0.999);
+    }
+    for (int pb = 0; pb < np; pb += kTrainThreads) {
+      const int cnt = min(kTrainThreads, np - pb);
+      int sh = 4;  // cnt <= 2^sh <= kTrainThreads
+      while ((1 << sh) < cnt) sh++;
+      const int batch = kGather >> sh;  // tiles fetched at a time: kGather / kTrainThreads loads per thread
+      const int gp = tid & ((1 << sh) - 1), bt = tid >> sh;
+      const float* const src = part + p0 + pb + gp;
+      float g = 0.0f;
+      for (int b0 = 0; b0 < tiles; b0 += batch) {
+        const int nb = min(batch, tiles - b0);
+        float x[kGather / kTrainThreads];
+#pragma unroll
+        for (int u = 0; u < kGather / kTrainThreads; u++) {
+          const int b = bt + u * (kTrainThreads >> sh);
+          x[u] = gp < cnt && b < nb ? __ldcg(src + (int64_t)(b0 + b) * (NP + 1)) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < kGather / kTrainThreads; u++) sm.gather[((bt + u * (kTrainThreads >> sh)) << sh) + gp] = x[u];
+        __syncthreads();
+        if (tid < cnt)
+#pragma unroll 16
+          for (int b = 0; b < nb; b++) g += sm.gather[(b << sh) + tid];
+        __syncthreads();
+      }
+      const int p = p0 + pb + tid;
+      if (tid < cnt) {
+        if (!update) {
+          grad[p] = p == NP ? g / (float)n : g;
+        } else if (p < NP) {
+          const float c1 = (float)__dsub_rn(1.0, b1k), c2 = (float)__dsub_rn(1.0, b2k);
+          const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+          if (!own) {
+            mp = m[p];
+            vp = v[p];
+            pp = params[p];
+          }
+          const float mm = b1 * mp + (1.0f - b1) * g;
+          const float vv = b2 * vp + (1.0f - b2) * g * g;
+          pp -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+          m[p] = mp = mm;
+          v[p] = vp = vv;
+          params[p] = pp;
+        }
+      }
+    }
+    if (it + 1 < total && !grid_barrier(sync, (unsigned)(2 * it + 2) * G)) return;
+  }
 }
 
 uint64_t splitmix64(uint64_t& s) {
@@ -183,7 +425,9 @@ double normal(uint64_t& s) {  // Box-Muller on two 53-bit uniforms
 struct bsmm_mlp_s {
   Norm norm{};
   int64_t step = 0;
-  DevBuf params, m, v, grad, part;
+  // params, m, v (kNPpad floats each), grad (NP + 1, padded alike) and the barrier's words in
+  // one allocation, owned by params
+  DevBuf params, m, v, grad, sync, part;
 };
 
 namespace {
@@ -203,24 +447,40 @@ bsmm_status mlp_alloc(DevBuf& b, size_t bytes) {
   return BSMM_OK;
 }
 
-size_t grad_smem() { return sizeof(float) * (NP + TILE * F + 4 * TILE * H + 2 * TILE); }
-
-bsmm_status loss_grad(bsmm_mlp_s* mlp, const float* X, const float* t, int64_t n, cudaStream_t st) {
-  const int nb = (int)((n + TILE - 1) / TILE);
-  bsmm_status s = mlp_alloc(mlp->part, sizeof(float) * (size_t)nb * (NP + 1));
+// `total` passes over the samples, the first `updates` of them Adam steps (see
+// mlp_train_kernel). The grid's CTAs wait for one another, so the launch is cooperative and
+// no larger than what is resident at once.
+bsmm_status train(bsmm_mlp_s* mlp, const float* X, const float* t, int64_t n, int total, int updates, float lr,
+                  cudaStream_t st) {
+  const int64_t tiles64 = (n + TILE - 1) / TILE;
+  if (tiles64 > (1 << 30)) return set_error("too many samples"), BSMM_ERR_INVALID;
+  int tiles = (int)tiles64;
+  const bsmm_status s = mlp_alloc(mlp->part, sizeof(float) * (size_t)tiles * (NP + 1));
   if (s != BSMM_OK) return s;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem()) !=
-        cudaSuccess)
-      return set_error("cudaFuncSetAttribute failed"), BSMM_ERR_CUDA;
-    attr = true;
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainShared));
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_kernel, kTrainThreads, sizeof(TrainShared));
+  if (e == cudaSuccess) e = cudaMemsetAsync(mlp->sync.p, 0, 2 * sizeof(unsigned), st);
+  if (e == cudaSuccess) {
+    const int grid = std::max(1, std::min(tiles, sms * std::max(1, per_sm)));
+    float *params = (float*)mlp->params.p, *m = (float*)mlp->m.p, *v = (float*)mlp->v.p, *grad = (float*)mlp->grad.p;
+    float* part = (float*)mlp->part.p;
+    unsigned* sync = (unsigned*)mlp->sync.p;
+    void* args[] = {&params, &m, &v, &grad, &part, &mlp->norm, &X, &t, &n, &tiles, &total, &updates, &lr, &sync};
+    e = cudaLaunchCooperativeKernel((const void*)mlp_train_kernel, dim3(grid), dim3(kTrainThreads), args,
+                                    sizeof(TrainShared), st);
   }
-  mlp_grad_kernel<<<nb, TILE, grad_smem(), st>>>((const float*)mlp->params.p, mlp->norm, X, t, n,
-                                                 (float*)mlp->part.p);
-  mlp_reduce_kernel<<<(NP + 1 + 255) / 256, 256, 0, st>>>((const float*)mlp->part.p, nb, n, (float*)mlp->grad.p);
-  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(std::string("mlp kernels: ") + cudaGetErrorString(e)), BSMM_ERR_CUDA;
+  return BSMM_OK;
+}
+
+// After a copy of the launch's outputs has been waited for: did a grid barrier run out?
+bsmm_status barrier_status(unsigned flag) {
+  if (flag) return set_error("mlp training: a grid barrier timed out"), BSMM_ERR_TIMEOUT;
   return BSMM_OK;
 }
 
@@ -244,15 +504,19 @@ bsmm_status bsmm_mlp_create(bsmm_mlp_t* out, uint64_t seed) {
   }
   mlp->norm.ymu = 0.0f;
   mlp->norm.ysd = 1.0f;
-  bsmm_status st;
-  if ((st = mlp_alloc(mlp->params, sizeof(float) * NP)) != BSMM_OK || (st = mlp_alloc(mlp->m, sizeof(float) * NP)) != BSMM_OK ||
-      (st = mlp_alloc(mlp->v, sizeof(float) * NP)) != BSMM_OK ||
-      (st = mlp_alloc(mlp->grad, sizeof(float) * (NP + 1))) != BSMM_OK) {
+  constexpr size_t kArray = sizeof(float) * (kNPpad + 4);
+  const bsmm_status st = mlp_alloc(mlp->params, 4 * kArray + 16);
+  if (st != BSMM_OK) {
     bsmm_mlp_destroy(mlp);
     return st;
   }
-  if (cudaMemcpy(mlp->params.p, p.data(), sizeof(float) * NP, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(mlp->m.p, 0, sizeof(float) * NP) != cudaSuccess || cudaMemset(mlp->v.p, 0, sizeof(float) * NP) != cudaSuccess) {
+  unsigned char* const base = (unsigned char*)mlp->params.p;
+  mlp->m.p = base + kArray;
+  mlp->v.p = base + 2 * kArray;
+  mlp->grad.p = base + 3 * kArray;
+  mlp->sync.p = base + 4 * kArray;
+  if (cudaMemset(mlp->params.p, 0, 4 * kArray + 16) != cudaSuccess ||
+      cudaMemcpy(mlp->params.p, p.data(), sizeof(float) * NP, cudaMemcpyHostToDevice) != cudaSuccess) {
     bsmm_mlp_destroy(mlp);
     return set_error("mlp initialisation copy failed"), BSMM_ERR_CUDA;
   }
@@ -303,12 +567,15 @@ bsmm_status bsmm_mlp_loss_grad(bsmm_mlp_t mlp, const float* X, const float* t, i
                                void* stream) {
   if (!mlp || !X || !t || n <= 0) return set_error("bad arguments"), BSMM_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  bsmm_status s = loss_grad(mlp, X, t, n, st);
+  bsmm_status s = train(mlp, X, t, n, 1, 0, 0.0f, st);
   if (s != BSMM_OK) return s;
   std::vector<float> g(NP + 1);
+  unsigned flag = 0;
   if (cudaMemcpyAsync(g.data(), mlp->grad.p, sizeof(float) * (NP + 1), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaMemcpyAsync(&flag, (unsigned*)mlp->sync.p + 1, sizeof(flag), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return set_error("copy failed"), BSMM_ERR_CUDA;
+  if ((s = barrier_status(flag)) != BSMM_OK) return s;
   if (loss) *loss = g[NP];
   if (grad) std::memcpy(grad, g.data(), sizeof(float) * NP);
   return BSMM_OK;
@@ -324,14 +591,19 @@ bsmm_status bsmm_mlp_fit(bsmm_mlp_t mlp, const float* X, const float* t, int64_t
       cudaMemcpyAsync(ht.data(), t, sizeof(float) * ht.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return set_error("copy failed"), BSMM_ERR_CUDA;
-  for (int f = 0; f < F; f++) {
-    double s1 = 0, s2 = 0;
-    for (int64_t i = 0; i < n; i++) s1 += hx[i * F + f];
-    const double mu = s1 / n;
-    for (int64_t i = 0; i < n; i++) s2 += (hx[i * F + f] - mu) * (hx[i * F + f] - mu);
-    const double sd = std::sqrt(s2 / n);
-    mlp->norm.xmu[f] = (float)mu;
-    mlp->norm.xsd[f] = sd > 0 ? (float)sd : 1.0f;
+  {
+    // (the features side by side: their sums are independent chains, each in sample order)
+    double s1[F] = {}, s2[F] = {}, mu[F];
+    for (int64_t i = 0; i < n; i++)
+      for (int f = 0; f < F; f++) s1[f] += hx[i * F + f];
+    for (int f = 0; f < F; f++) mu[f] = s1[f] / n;
+    for (int64_t i = 0; i < n; i++)
+      for (int f = 0; f < F; f++) s2[f] += (hx[i * F + f] - mu[f]) * (hx[i * F + f] - mu[f]);
+    for (int f = 0; f < F; f++) {
+      const double sd = std::sqrt(s2[f] / n);
+      mlp->norm.xmu[f] = (float)mu[f];
+      mlp->norm.xsd[f] = sd > 0 ? (float)sd : 1.0f;
+    }
   }
   {
     double s1 = 0, s2 = 0;
@@ -345,23 +617,18 @@ bsmm_status bsmm_mlp_fit(bsmm_mlp_t mlp, const float* X, const float* t, int64_t
   if (cudaMemsetAsync(mlp->m.p, 0, sizeof(float) * NP, st) != cudaSuccess ||
       cudaMemsetAsync(mlp->v.p, 0, sizeof(float) * NP, st) != cudaSuccess)
     return set_error("memset failed"), BSMM_ERR_CUDA;
-  double c1 = 1.0, c2 = 1.0;
-  for (int32_t k = 1; k <= steps; k++) {
-    bsmm_status s = loss_grad(mlp, X, t, n, st);
+  const int total = steps + (final_loss ? 1 : 0);
+  if (total > 0) {
+    bsmm_status s = train(mlp, X, t, n, total, steps, lr, st);
     if (s != BSMM_OK) return s;
-    c1 *= 0.9;
-    c2 *= 0.999;
-    mlp_adam_kernel<<<(NP + 255) / 256, 256, 0, st>>>((float*)mlp->params.p, (float*)mlp->m.p, (float*)mlp->v.p,
-                                                       (const float*)mlp->grad.p, lr, (float)(1.0 - c1),
-                                                       (float)(1.0 - c2));
   }
-  if (cudaGetLastError() != cudaSuccess) return set_error("adam kernel failed"), BSMM_ERR_CUDA;
   if (final_loss) {
-    bsmm_status s = loss_grad(mlp, X, t, n, st);
-    if (s != BSMM_OK) return s;
+    unsigned flag = 0;
     if (cudaMemcpyAsync(final_loss, (float*)mlp->grad.p + NP, sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&flag, (unsigned*)mlp->sync.p + 1, sizeof(flag), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
       return set_error("copy failed"), BSMM_ERR_CUDA;
+    return barrier_status(flag);
   }
   return BSMM_OK;
 }
@@ -516,7 +783,7 @@ bsmm_status bsmm_mlp_load(bsmm_mlp_t* out, const char* path) {
 
 void bsmm_mlp_destroy(bsmm_mlp_t mlp) {
   if (!mlp) return;
-  for (DevBuf* b : {&mlp->params, &mlp->m, &mlp->v, &mlp->grad, &mlp->part})
+  for (DevBuf* b : {&mlp->params, &mlp->part})
     if (b->p) cudaFree(b->p);
   delete mlp;
 }
