@@ -169,8 +169,11 @@ def kernel_source_hash():
     """Hash of the contraction kernel's sources with comments and blank space removed, so a
     comment-only edit keeps the recorded DRAM counters valid and a code edit does not."""
     h = hashlib.sha256()
-    for f in ("split.cu", "bsmm_internal.h"):
-        with open(os.path.join(ROOT, "paper_1504_05046_gb300", "csrc", f)) as fh:
+    for f in ("split.cu", "split_device.cuh", "wide.cu", "bsmm_internal.h"):
+        path = os.path.join(ROOT, "paper_1504_05046_gb300", "csrc", f)
+        if not os.path.exists(path):
+            continue
+        with open(path) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
         src = re.sub(r"//[^\n]*", "", src)
