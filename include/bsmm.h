@@ -95,7 +95,12 @@ typedef struct {
                               -1 = the planner's choice: 4, else 2, when the column blocks of
                               every group carry the same tensor-core work to within 0.5% (a
                               dense block pattern), else 1. Plans of one batch need equal
-                              sizes, so a plan meant for a batch should fix it. */
+                              sizes, so a plan meant for a batch should fix it.
+                              A plan with groups of 2 or 4, 3 or more slices, a dense block
+                              pattern (each pair of column blocks has B tiles at the same
+                              inner blocks) and a deep inner sum (3072 elements or so) runs its
+                              own executes with CTAs of two column blocks each: half as many
+                              CTAs per group, the same work units, the same result bits. */
   int32_t fp64_tile;       /* FP64 mode: sub-tile edge of a work unit, 32 or 64 (0 = 32) */
   int32_t stages;          /* split modes: depth of the shared-memory ring of 32-deep k chunks
                               (k panels in flight), 2..8 and within the 227 KB shared memory of
@@ -522,7 +527,8 @@ bsmm_status bsmm_plan_cost_source(bsmm_plan_t plan, int32_t* source);
 /*
  * The contraction launch the planner chose for a plan (host outputs; any may be NULL):
  * cluster = CTAs per column-block group (1, 2 or 4; bsmm_options.cluster = -1 resolved),
- * store_warps = 1 when the kernel form has C store warps, epi_walk = 1 when the epilogue
+ * store_warps = 1 when the kernel form has C store warps (0 also for the form with two column
+ * blocks per CTA, see bsmm_options.cluster), epi_walk = 1 when the epilogue
  * walks its own k lists for the accumulation groups (long k lists, 3 to 6 slices with
  * store warps) rather than taking the MMA warps' descriptors, stages = depth of the
  * shared-memory ring, ctas = persistent CTAs (FP64) or groups (split modes) of a launch.

@@ -26,6 +26,10 @@ constexpr int kSplitMaxS = 6;      // slices per operand
 constexpr int kSplitEpiWarps = 8;  // epilogue warps (2 per TMEM lane quadrant)
 constexpr int kSplitGuard = 55;    // guard bits of the 128-bit accumulator below the largest scale
 constexpr double kEpiWalkBlocks = 32.0;  // mean k blocks per unit from which the epilogue walks
+// mean inner depth of a unit from which the 64-column form is taken: with many units per
+// group of CTAs, and always
+constexpr double kWideDepthMany = 2048.0, kWideDepth = 3072.0;
+constexpr int64_t kWideManyUnits = 8;
 constexpr int kSplitMaxK = 8192;   // inner blocks per product
 constexpr int64_t kSplitMaxInner = int64_t(1) << 22;  // inner elements per product (128-bit sums' headroom)
 
@@ -125,6 +129,8 @@ struct SplitArgs {
   int32_t cl, CBG;          // CTAs per column-block group; groups (units are (rb, group))
   int32_t sw;               // the contraction kernel's form: 1 = with C store warps
   int32_t deep;             // 1: some inner block is deeper than kdepth (the kernel's DEEP form)
+  int32_t wide, wstages;    // 1: a plan of its own runs in the 64-column form (wide.cu) with this ring
+                            // depth; its groups are then of cl/2 CTAs, two column blocks each
   int32_t epi_walk;         // 1: the epilogue finds the accumulation groups on its own k list
                             // (long lists); 0: it takes them from the MMA warps' descriptors
   int64_t Mtot, Ntot;
@@ -230,6 +236,10 @@ cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEven
 cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* ev, int* k);
 int split_prep_kernels(const SplitArgs& a);  // how many kernels launch_split_prep launches
 cudaError_t launch_split_mma(const SplitArgs& a, int clusters, cudaStream_t st);
+// the 64-column form (wide.cu): `groups` of a.cl/2 CTAs
+cudaError_t launch_split_wide(const SplitArgs& a, int groups, cudaStream_t st);
+int split_wide_stages(int s);  // its deepest ring
+size_t split_wide_smem_bytes(int s, int stages);
 // split k: the reductions of the regions whose k-list was split (no launch when none)
 cudaError_t launch_split_reduce(const SplitArgs& a, cudaStream_t st);
 // a kernel whose bounded waits can never be satisfied (see bsmm_selftest_wait)
@@ -305,6 +315,7 @@ struct bsmm_plan_s {
   int sw = 0;                // contraction kernel with C store warps
   int epi_walk = 0;          // the epilogue walks the k lists itself (SplitArgs::epi_walk)
   int32_t qmax = 0;          // the largest inner block
+  int wide = 0, wstages = 0; // the contraction runs in the 64-column form (SplitArgs::wide)
   int deep = 0;              // some inner block is deeper than the exact FP32 depth
   int64_t Mtot = 0, Ntot = 0, colexp_ld = 0;
   int64_t apk_bytes = 0, bpk_bytes = 0;

@@ -117,7 +117,8 @@ int machine_bins(const bsmm_plan_s* p) {
   if (p->opt.mode == BSMM_FP64)
     c = (int64_t)p->sms * std::max(1, fp64_ctas_per_sm(p->f64_tile));
   else
-    c = std::max(1, split_max_clusters(p->s, p->cl, p->stages, p->sw != 0));
+    c = p->wide ? std::max(1, p->sms / (p->cl / 2))  // one CTA per SM, two column blocks each
+                : std::max(1, split_max_clusters(p->s, p->cl, p->stages, p->sw != 0));
   if (p->opt.max_ctas > 0) c = std::min<int64_t>(c, p->opt.max_ctas);
   return (int)std::max<int64_t>(1, c);
 }
@@ -584,6 +585,27 @@ bsmm_status plan_split(bsmm_plan_s* p) {
     double blocks = 0.0;
     for (size_t u = 0; u < base.size(); u++) blocks += (double)blen[u];
     p->epi_walk = !base.empty() && blocks >= kEpiWalkBlocks * (double)base.size() ? 1 : 0;
+  }
+  // The 64-column form (wide.cu): groups of several column blocks whose pairs carry the same
+  // inner blocks, and k lists deep enough that what it does not overlap (a unit's first and
+  // last group, and with 5 and 6 slices the drain of every group) is a small part. Measured
+  // contraction times, 32-column form against this one:
+  //   6 slices, dense n = 2048: 290 / 324 us, 2560: 553 / 568, 3072: 970 / 888, 4096: 2214 /
+  //   1979, 6144: 7188 / 6290, 16384: 133.1 / 112.3 ms; Bernoulli(0.5) masks, 8192 (2048 deep,
+  //   54 units per group): 3970 / 3820; 512 x 32768 deep: 331 / 269
+  //   4 slices: 202 / 214, 375 / 363, 646 / 575, 1488 / 1296, 4953 / 4126; 2563 / 2337; 238 / 204
+  p->wide = 0;
+  if (CL >= 2 && s >= 3 && p->sw && !p->deep && !base.empty()) {
+    bool pairs = true;
+    for (int cb = 0; cb + 1 < CB && pairs; cb += 2)
+      for (int wd = 0; wd < KW && pairs; wd++) pairs = presB[(size_t)cb * KW + wd] == presB[(size_t)(cb + 1) * KW + wd];
+    double depth = 0.0;
+    for (int32_t k : bk) depth += p->q[k];
+    depth /= (double)base.size();
+    const bool many = (int64_t)base.size() >= kWideManyUnits * (p->sms / (CL / 2));
+    p->wide = pairs && depth >= (many ? kWideDepthMany : kWideDepth) ? 1 : 0;
+    const int deepest = split_wide_stages(s);
+    p->wstages = p->opt.stages ? std::min(p->opt.stages, deepest) : deepest;
   }
   const std::vector<int32_t> np =
       choose_pieces(bcost, blen, machine_bins(p), kSplitPieceOverhead, p->opt.ksplit == -1 ? 0 : p->opt.ksplit);
@@ -1087,9 +1109,9 @@ bsmm_status bsmm_plan_form(bsmm_plan_t p, int32_t* cluster, int32_t* store_warps
   if (!p) return set_error("plan is NULL"), BSMM_ERR_INVALID;
   const bool split = p->opt.mode != BSMM_FP64;
   if (cluster) *cluster = split ? p->cl : 1;
-  if (store_warps) *store_warps = split ? p->sw : 0;
-  if (epi_walk) *epi_walk = split && p->sw && p->s >= 3 ? p->epi_walk : 0;
-  if (stages) *stages = split ? p->stages : 0;
+  if (store_warps) *store_warps = split && !p->wide ? p->sw : 0;
+  if (epi_walk) *epi_walk = split && p->sw && p->s >= 3 ? p->epi_walk || p->wide : 0;
+  if (stages) *stages = split ? (p->wide ? p->wstages : p->stages) : 0;
   if (ctas) *ctas = p->ctas;
   return BSMM_OK;
 }

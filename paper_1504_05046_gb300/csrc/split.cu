@@ -483,14 +483,7 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
           }
 #pragma unroll
           for (int c = 0; c < CW; c++) {
-            // T = sum_d S_d 2^(7(S+1-d)), exact: the tensor core's FP32 sums are integers
-            long long T = 0;
-#pragma unroll
-            for (int d = 0; d < S; d++) {
-              int iv;
-              asm("cvt.rni.s32.f32 %0, %1;" : "=r"(iv) : "f"(__uint_as_float(v[d][c])));
-              T += (long long)iv * (1ll << (kSplitBeta * (S - 1 - d)));
-            }
+            const long long T = diagonal_sum<S, CW, false>(v, c);  // exact: the tensor core's FP32 sums are integers
             const int col = cc * CW + c;  // column within this thread's TH
             const uint4& w4 = cx[col >> 3];
             const int e = col & 7;
@@ -627,7 +620,8 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const __grid_constant
     unsigned long long v = 0ull;
     if (row_ok && n < a.Ntot) {
       const int L = Lrow + (a.rowscale ? a.eBmaxc[n] : a.eBmax[a.col_tile[n]]);
-      v = a.f32 ? acc_to_float(w[c], L) : acc_to_double(w[c], L);
+      v = a.f32 ? acc_bits_any<true>(w[c][0], w[c][1], w[c][2], w[c][3], L)
+                : acc_bits_any<false>(w[c][0], w[c][1], w[c][2], w[c][3], L);
     }
     cstage[lane * (TN + 1) + warp * kCols + c] = v;
   }
@@ -727,7 +721,7 @@ cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEven
   nvtxRangePop();
   if (e != cudaSuccess) return e;
   nvtxRangePushA("bsmm split: contraction");
-  e = launch_split_mma(a, ctas, st);
+  e = a.wide && !a.prods ? launch_split_wide(a, ctas, st) : launch_split_mma(a, ctas, st);
   nvtxRangePop();
   if (ev) cudaEventRecord(ev[++k], st);
   if (e == cudaSuccess && !a.prods && a.n_red > 0) {  // a batch launches its products' reductions

@@ -177,6 +177,46 @@ __device__ __forceinline__ uint32_t idesc_f16(int M, int N, bool fp16) {
 }
 
 // ---------------------------------------------------------------- exact accumulation
+// The exact integer of an element's accumulation group from its diagonal sums (integers of
+// magnitude <= 2^24 as floats): T = sum_d S_d 2^(7(S-1-d)), |T| < 2^59.
+// Bound by the float-to-integer conversions: 16 lanes per clock and SM, so six of them hold
+// two warps of a scheduler for 96 cycles, and all else an element needs fits beside them.
+// Two neighbouring diagonals a, b are therefore joined into a 2^7 + b (below 2^31 from 3
+// slices on) with one conversion where kMagic: b's part above 7 bits moves over to a (both
+// exact: |a| <= 2^24 (S+1)/(S+2), the carry <= 2^17), and the small rest is read off the bits
+// of rest + 1.5 2^23. Two of the three joins of 6 slices that way balance the conversions
+// with the other instructions: 112 to 90 cycles per element of two warps (128 when every
+// diagonal was converted and shifted on its own).
+__device__ __forceinline__ int to_int(float x) {  // an integer's value
+  int r;
+  asm("cvt.rni.s32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return r;
+}
+template <bool kMagic>
+__device__ __forceinline__ int join_pair(float a, float b) {
+  if constexpr (!kMagic) return to_int(a) * 128 + to_int(b);
+  constexpr float kM = 12582912.0f;                     // 1.5 2^23: adding it rounds to an integer
+  const float h = fmaf(b, 1.0f / 128, kM) - kM;         // the carry into a
+  const float rest = fmaf(h, -128.0f, b);               // |rest| <= 64
+  return to_int(a + h) * 128 + (__float_as_int(rest + kM) - __float_as_int(kM));
+}
+template <int S, int CW, bool kMagic>
+__device__ __forceinline__ long long diagonal_sum(const uint32_t (&v)[S][CW], int c) {
+  auto f = [&](int d) { return __uint_as_float(v[d][c]); };
+  if constexpr (S == 1) {
+    return to_int(f(0));
+  } else if constexpr (S == 2) {
+    return (long long)to_int(f(0)) * 128 + to_int(f(1));
+  } else {
+    long long T = join_pair<kMagic>(f(S - 2), f(S - 1));
+    if constexpr (S >= 4) T += (long long)join_pair<kMagic && (S >= 5)>(f(S - 4), f(S - 3)) * (1ll << 14);
+    if constexpr (S == 3) T += (long long)to_int(f(0)) * (1ll << 14);
+    if constexpr (S == 5) T += (long long)to_int(f(0)) * (1ll << 28);
+    if constexpr (S == 6) T += (long long)join_pair<false>(f(0), f(1)) * (1ll << 28);
+    return T;
+  }
+}
+
 // w (four 32-bit words, two's complement) += T * 2^sh, with floor(T / 2^-sh) for sh < 0.
 // |T| < 2^59 and sh <= kSplitGuard for every accumulation group (its depth keeps each FP32
 // partial sum below 2^24); an absent tile pair has T = 0.
@@ -195,6 +235,27 @@ __device__ __forceinline__ void acc_add(uint32_t (&w)[4], long long T, int sh) {
       : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
       : "r"((uint32_t)lo), "r"((uint32_t)((unsigned long long)lo >> 32)), "r"((uint32_t)hi),
         "r"((uint32_t)((unsigned long long)hi >> 32)));
+}
+
+// w += T
+__device__ __forceinline__ void acc_add_plain(uint32_t (&w)[4], long long T) {
+  const uint32_t s = (uint32_t)(T >> 63);
+  asm("add.cc.u32 %0, %0, %4;\n\t"
+      "addc.cc.u32 %1, %1, %5;\n\t"
+      "addc.cc.u32 %2, %2, %6;\n\t"
+      "addc.u32 %3, %3, %6;"
+      : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
+      : "r"((uint32_t)T), "r"((uint32_t)((unsigned long long)T >> 32)), "r"(s));
+}
+
+// w *= 2^sh (0 <= sh < 64)
+__device__ __forceinline__ void acc_shl(uint32_t (&w)[4], int sh) {
+  const bool word = sh >= 32;
+  const uint32_t w3 = word ? w[2] : w[3], w2 = word ? w[1] : w[2], w1 = word ? w[0] : w[1], w0 = word ? 0u : w[0];
+  w[3] = __funnelshift_l(w2, w3, sh);  // (shifts by sh mod 32)
+  w[2] = __funnelshift_l(w1, w2, sh);
+  w[1] = __funnelshift_l(w0, w1, sh);
+  w[0] = __funnelshift_l(0u, w0, sh);
 }
 
 // 64-bit window of a 128-bit magnitude shifted right by r (0 <= r < 128)
@@ -276,38 +337,51 @@ __device__ __noinline__ unsigned long long acc_round_subnormal(uint32_t w0, uint
   return q;
 }
 
-// The integer w times 2^L rounded to the nearest double: the 53-bit significand and the
-// exponent are assembled into the double's bit pattern (GB300's FP64 pipe is narrow, so
-// no FP64 instruction is spent per element). A result below the normal range is rounded
+// The integer w times 2^L rounded to the nearest double, as its bits: the 53-bit significand
+// and the exponent are assembled into the double's bit pattern (GB300's FP64 pipe is narrow,
+// so no FP64 instruction is spent per element). A result below the normal range is rounded
 // once on the subnormal grid (not first to 53 bits); one beyond it is an infinity.
 // The significand with its leading one is added to the exponent field less one, so a
 // rounding that carries out of it moves the exponent (and 2046 to an infinity) by itself.
-// Branch-free but for the two rare ranges: a unit's 16 sums per thread take 4400 cycles
-// (banded 32768 product), 11700 when every sum chose among shift cases by branches.
-__device__ __forceinline__ unsigned long long acc_to_double(const uint32_t (&w)[4], int L) {
+// No branch, so that a thread's values overlap: the two rare ranges set `rare` (the value
+// returned is then not the result) and are formed by acc_bits_any. A unit's 16 sums per
+// thread took 11700 cycles when every sum chose among shift cases by branches (banded 32768
+// product), 4400 with only the rare ranges branching.
+template <bool F32>
+__device__ __forceinline__ unsigned long long acc_bits(const uint32_t (&w)[4], int L, bool& rare) {
   uint32_t t[3];
-  const int biased = acc_normalise(w, t) + L + 1023;
-  const unsigned long long sign = (unsigned long long)(w[3] & 0x80000000u) << 32;
-  if (t[0] == 0u) return 0ull;
-  if (biased < 1) return sign | acc_round_subnormal<53>(w[0], w[1], w[2], w[3], L, -1074);
-  if (biased > 2046) return sign | 0x7FF0000000000000ull;
-  const unsigned long long mant = (((unsigned long long)t[0] << 32) | t[1]) >> 11;  // 53 bits
-  const uint32_t low = (t[1] & 0x3FFu) | t[2];
-  const uint32_t inc = (t[1] >> 10) & 1u & ((low != 0u ? 1u : 0u) | (t[1] >> 11));
-  return (sign | ((unsigned long long)(uint32_t)(biased - 1) << 52)) + mant + inc;
-}
-
-// The same rounded once to float32 (24-bit significand), for float32 elements.
-__device__ __forceinline__ uint32_t acc_to_float(const uint32_t (&w)[4], int L) {
-  uint32_t t[3];
-  const int biased = acc_normalise(w, t) + L + 127;
+  const int msb = acc_normalise(w, t);
   const uint32_t sign = w[3] & 0x80000000u;
-  if (t[0] == 0u) return 0u;
-  if (biased < 1) return sign | (uint32_t)acc_round_subnormal<24>(w[0], w[1], w[2], w[3], L, -149);
-  if (biased > 254) return sign | 0x7F800000u;
-  const uint32_t low = (t[0] & 0x7Fu) | t[1] | t[2];
-  const uint32_t inc = (t[0] >> 7) & 1u & ((low != 0u ? 1u : 0u) | (t[0] >> 8));
-  return (sign | ((uint32_t)(biased - 1) << 23)) + (t[0] >> 8) + inc;
+  const bool nonzero = t[0] != 0u;
+  if constexpr (F32) {  // 24-bit significand
+    const int biased = msb + L + 127;
+    rare |= nonzero && (uint32_t)(biased - 1) > 253u;
+    const uint32_t low = (t[0] & 0x7Fu) | t[1] | t[2];
+    const uint32_t inc = (t[0] >> 7) & 1u & ((low != 0u ? 1u : 0u) | (t[0] >> 8));
+    const uint32_t v = (sign | ((uint32_t)(biased - 1) << 23)) + (t[0] >> 8) + inc;
+    return nonzero ? v : 0u;
+  } else {
+    const int biased = msb + L + 1023;
+    rare |= nonzero && (uint32_t)(biased - 1) > 2045u;
+    const unsigned long long mant = (((unsigned long long)t[0] << 32) | t[1]) >> 11;
+    const uint32_t low = (t[1] & 0x3FFu) | t[2];
+    const uint32_t inc = (t[1] >> 10) & 1u & ((low != 0u ? 1u : 0u) | (t[1] >> 11));
+    const unsigned long long v =
+        ((unsigned long long)(sign | ((uint32_t)(biased - 1) << 20)) << 32) + mant + inc;
+    return nonzero ? v : 0ull;
+  }
+}
+template <bool F32>
+__device__ __noinline__ unsigned long long acc_bits_any(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, int L) {
+  const uint32_t w[4] = {w0, w1, w2, w3};
+  bool rare = false;
+  const unsigned long long v = acc_bits<F32>(w, L, rare);
+  if (!rare) return v;
+  uint32_t t[3];
+  const int biased = acc_normalise(w, t) + L + (F32 ? 127 : 1023);
+  const unsigned long long sign = F32 ? (w3 & 0x80000000u) : (unsigned long long)(w3 & 0x80000000u) << 32;
+  if (biased > 0) return sign | (F32 ? 0x7F800000ull : 0x7FF0000000000000ull);
+  return sign | (F32 ? acc_round_subnormal<24>(w0, w1, w2, w3, L, -149) : acc_round_subnormal<53>(w0, w1, w2, w3, L, -1074));
 }
 
 // w += v, 128-bit two's complement
@@ -515,9 +589,16 @@ __device__ __forceinline__ void load_emaxc(const SplitArgs& P, int64_t n0, int (
 template <int TH, bool F32>
 __device__ __forceinline__ void round_row(const uint32_t (&acc)[TH][4], unsigned long long* srow,
                                           const int (&emc)[TH], int Lrow) {
+  bool rare = false;
 #pragma unroll
-  for (int c = 0; c < TH; c++) srow[c] = F32 ? acc_to_float(acc[c], Lrow + emc[c]) : acc_to_double(acc[c], Lrow + emc[c]);
+  for (int c = 0; c < TH; c++) srow[c] = acc_bits<F32>(acc[c], Lrow + emc[c], rare);
+  if (rare) {
+#pragma unroll
+    for (int c = 0; c < TH; c++)
+      srow[c] = acc_bits_any<F32>(acc[c][0], acc[c][1], acc[c][2], acc[c][3], Lrow + emc[c]);
+  }
 }
+
 
 // ---------------------------------------------------------------- kernel 3: contraction
 // Ascending k blocks of one unit (a 128-row block times a group of cl column blocks):
