@@ -74,7 +74,9 @@ typedef enum {
 } bsmm_elem;
 
 typedef enum {
-  BSMM_SCHED_FLOPS = 0,   /* order and pack work units by useful flop count */
+  BSMM_SCHED_FLOPS = 0,   /* order and pack work units by the planner's own costs: useful flop
+                             counts in FP64 mode, the executed work (a fixed part plus the
+                             32-deep chunks of the unit's k-list) in the split modes */
   BSMM_SCHED_COSTS = 1,   /* by costs given through bsmm_plan_set_costs (e.g. the MLP) */
   BSMM_SCHED_NATURAL = 2  /* no reordering: units in row-major order, dealt round robin */
 } bsmm_schedule;
@@ -180,7 +182,7 @@ typedef struct {
 } bsmm_options;
 
 typedef enum {
-  BSMM_COSTS_FLOPS = 0,  /* useful flop counts (the default, and the model file's fallback) */
+  BSMM_COSTS_FLOPS = 0,  /* the planner's own, see BSMM_SCHED_FLOPS (the default, and the model file's fallback) */
   BSMM_COSTS_MODEL = 1,  /* predicted by the cost-model file of bsmm_options.model_path */
   BSMM_COSTS_GIVEN = 2   /* set by bsmm_plan_set_costs or bsmm_plan_predict_costs */
 } bsmm_cost_source;

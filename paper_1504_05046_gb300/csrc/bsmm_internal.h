@@ -306,6 +306,7 @@ struct bsmm_plan_s {
   std::vector<int32_t> unit_pieces;  // per unit: pieces of its region (1: not split)
   int64_t n_slots = 0;
   std::vector<double> flop_cost, cost;
+  std::vector<double> unit_cost;  // split modes: the planner's estimate of the units' times
   std::vector<float> features;  // n_units x BSMM_NFEATURES
   int ctas = 0;
   std::vector<int32_t> sched_ptr, sched_units;

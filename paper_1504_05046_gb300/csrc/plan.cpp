@@ -672,6 +672,13 @@ bsmm_status plan_split(bsmm_plan_s* p) {
         if (g_r > kg || (g_r == kg && q_r > kq)) kq = q_r, kg = g_r, kc = c_r, nk = n_r;
       }
       p->flop_cost.push_back(std::max(fl, 1.0));
+      // What the unit costs the packing: nanoseconds, as measured unit times have it (least
+      // squares over a clustered, a banded and a Bernoulli product, 3, 4 and 6 slices: 2100 to
+      // 3000 ns per unit and 311, 325 and 517 to 650 ns per 32-deep chunk of its slowest CTA).
+      // Useful flops leave out absent tiles inside the 128-row block, padding and the fixed
+      // part, by different factors for every unit: on the clustered 24576 product the CTAs'
+      // loads then differ so much that the contraction takes 10.56 ms against 7.52 ms.
+      p->unit_cost.push_back(2500.0 + 100.0 * s * (double)kc);
       const double padded = 2.0 * kSplitBM * tn * CL * 16.0 * (double)kg;
       float f[BSMM_NFEATURES] = {lg((double)(m1 - m0)), lg((double)(n1 - n0)), lg((double)nk), lg((double)kq),
                                  lg((double)kg), lg(fl), (float)(padded > 0 ? fl / padded : 0.0),
@@ -947,7 +954,7 @@ bsmm_status plan_build(bsmm_plan_t* out, int32_t M, const int32_t* row_sizes, in
     return st;
   }
   p->donor = nullptr;  // only planning reads it
-  p->cost = p->flop_cost;
+  p->cost = p->unit_cost.empty() ? p->flop_cost : p->unit_cost;
   p->ctas = default_ctas(p);
   pack_lpt(p);
 
@@ -992,7 +999,7 @@ bsmm_status plan_build(bsmm_plan_t* out, int32_t M, const int32_t* row_sizes, in
       if (bsmm_plan_predict_costs(p, mlp, nullptr) == BSMM_OK) {
         p->cost_source = BSMM_COSTS_MODEL;
       } else {  // back to the flop-count packing
-        p->cost = p->flop_cost;
+        p->cost = p->unit_cost.empty() ? p->flop_cost : p->unit_cost;
         p->opt.schedule = o.schedule;
         pack_lpt(p);
         if ((st = upload_schedule(p)) != BSMM_OK) {
