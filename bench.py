@@ -35,13 +35,12 @@ sys.path.insert(0, ROOT)
 
 METRIC = "useful TFLOP/s (nonzero-tile flops) & % of peak; split vs FP64 at <=1e-11 rel err"
 PROFILE_FILE = os.path.join(ROOT, "profiles", "split_mma_kernel_nonuniform_dense.txt")
-# exponents, scales, scale classes, slices, contraction
 def kernels_per_execute(P, plan, mode, split_scale=0):
-    """Kernels one bsmm_execute launches: FP64 the tile kernel; split modes the exponent
-    (and line exponent), scale, class, pack and contraction kernels; plus the split-k
-    reduction when the plan cut a k-list."""
+    """Kernels one bsmm_execute launches: FP64 the tile kernel; split modes the exponent, pack
+    (with the scale classes) and contraction kernels, and with row/column scaling the line
+    scale kernel; plus the split-k reduction when the plan cut a k-list."""
     red = int(P.bsmm_plan_ksplit(plan)["n_regions"] > 0)
-    return (1 if mode == P.BSMM_FP64 else 5 + int(split_scale)) + red
+    return (1 if mode == P.BSMM_FP64 else 3 + int(split_scale)) + red
 
 
 def parse():

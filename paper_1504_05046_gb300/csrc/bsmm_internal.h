@@ -180,8 +180,6 @@ struct SplitArgs {
   int32_t* eBcol;
   int32_t* eAmaxr;
   int32_t* eBmaxc;
-  int32_t* eAmax;           // M: largest exponent of the stored A tiles of a row block
-  int32_t* eBmax;           // N
   int32_t* eA;              // M x K
   int32_t* eB;              // K x N
   const int32_t* a_tiles;   // present A tiles (i*K+k), count n_a_tiles
@@ -326,7 +324,7 @@ struct bsmm_plan_s {
   bsmm::DevBuf d_row_tile, d_col_tile, d_presA, d_presB, d_presBg, d_apk_off, d_bpk_off, d_apk, d_bpk;
   bsmm::DevBuf d_eArow, d_eBcol, d_eAmaxr, d_eBmaxc;
   bsmm::DevBuf d_rowadj, d_coladj, d_emaxr, d_emaxc;
-  bsmm::DevBuf d_am, d_bm, d_rowexp, d_colexp, d_urow, d_ucol, d_eA, d_eB, d_eAmax, d_eBmax, d_a_tiles, d_b_tiles, d_a_blocks, d_b_blocks;
+  bsmm::DevBuf d_am, d_bm, d_rowexp, d_colexp, d_urow, d_ucol, d_eA, d_eB, d_a_tiles, d_b_tiles, d_a_blocks, d_b_blocks;
   bsmm::DevBuf d_err, d_timings, d_unit_cta, d_part, d_red;
   int32_t n_a_tiles = 0, n_b_tiles = 0, n_a_blocks = 0, n_b_blocks = 0;
 

@@ -97,8 +97,6 @@ void fill_split_args(bsmm_plan_s* p, SplitArgs& a, double alpha, const void* A, 
   a.eBmaxc = (int32_t*)p->d_eBmaxc.p;
   a.eA = (int32_t*)p->d_eA.p;
   a.eB = (int32_t*)p->d_eB.p;
-  a.eAmax = (int32_t*)p->d_eAmax.p;
-  a.eBmax = (int32_t*)p->d_eBmax.p;
   a.a_tiles = (const int32_t*)p->d_a_tiles.p;
   a.b_tiles = (const int32_t*)p->d_b_tiles.p;
   a.n_a_tiles = p->n_a_tiles;

@@ -65,7 +65,7 @@ struct NaTables {
   alignas(16) int16_t colexp[kNaColLd + 64];
   alignas(16) int32_t emaxr[kNaMaxM];
   alignas(16) int32_t emaxc[kNaColLd + 64];
-  int32_t eA[1], eB[1], eAmax[1], eBmax[1];
+  int32_t eA[1], eB[1];
   int32_t a_tiles[1], b_tiles[1];
   int32_t a_blocks[kNaRB], b_blocks[kNaCB];
   SplitUnit units[kNaUnits];
@@ -202,8 +202,6 @@ extern "C" bsmm_status bsmm_split_tile_noalloc(int32_t m, int32_t n, int32_t k, 
   a.emaxc = t->emaxc;
   a.eA = t->eA;
   a.eB = t->eB;
-  a.eAmax = t->eAmax;
-  a.eBmax = t->eBmax;
   a.a_tiles = t->a_tiles;
   a.b_tiles = t->b_tiles;
   a.n_a_tiles = k > 0 ? 1 : 0;

@@ -65,8 +65,35 @@ __device__ __forceinline__ int exponent_above32(uint32_t m) {
   return -126 - (__clz((int)m) - 8);  // subnormal: leading one at bit 31 - clz
 }
 
-__global__ void __launch_bounds__(256) split_exp_kernel(SplitArgs a) {
-  const int b = blockIdx.x;
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t n;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return n;
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// v into rank 0's copy of a shared variable
+__device__ __forceinline__ void store_rank0(unsigned long long* p, unsigned long long v) {
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(addr) : "r"((uint32_t)__cvta_generic_to_shared(p)));
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+
+// Per stored tile, the exponent of its largest magnitude; a CTA per tile, or a cluster of
+// CTAs when the tiles alone would leave most SMs idle (a small product's time is this
+// kernel's latency: one CTA takes a 160 x 160 tile in 12 rounds of loads). Bound by HBM.
+constexpr int kExpThreads = 256;
+constexpr int kExpCluster = 8;  // CTAs of a cluster, at most
+constexpr int kExpResident = 4 * 152;  // CTAs that fill the machine
+__global__ void __launch_bounds__(kExpThreads) split_exp_kernel(const __grid_constant__ SplitArgs a) {
+  const int nz = (int)cluster_size(), z = (int)cluster_rank();
+  if (nz > 1) cluster_arrive();  // (waited for before rank 0's shared memory is written: it has started)
+  const int b = blockIdx.x / nz;
   const bool isA = b < a.n_a_tiles;
   const int t = isA ? a.a_tiles[b] : a.b_tiles[b - a.n_a_tiles];
   int rows, cols;
@@ -76,6 +103,8 @@ __global__ void __launch_bounds__(256) split_exp_kernel(SplitArgs a) {
   // tile holds r x q' doubles (q' = 2q), a B tile q' x c' / 2 (c' = 2c)
   const double* x = (isA ? a.A : a.B) + (off < 0 ? 0 : (a.cplx ? 2 * off : off));
   const int64_t n = (int64_t)rows * cols / (a.cplx && !isA ? 2 : 1);
+  const int first = z * kExpThreads + threadIdx.x, step = nz * kExpThreads;
+  constexpr int kU = 4;  // loads in flight
   // the largest magnitude as bits: at or above kInfBits when a NaN or infinity is there
   unsigned long long mx = 0;
   if (a.f32 && off >= 0) {
@@ -88,18 +117,16 @@ __global__ void __launch_bounds__(256) split_exp_kernel(SplitArgs a) {
     } else {
       const uint4* x4 = reinterpret_cast<const uint4*>(xf);
       const int64_t n4 = n >> 2;
-      const int64_t bd = blockDim.x;
-      for (int64_t e = threadIdx.x; e < n4; e += 4 * bd) {  // four loads in flight
-        uint4 v[4];
+      for (int64_t e = first; e < n4; e += kU * step) {
+        uint4 v[kU];
 #pragma unroll
-        for (int u = 0; u < 4; u++) v[u] = e + u * bd < n4 ? __ldg(x4 + e + u * bd) : make_uint4(0u, 0u, 0u, 0u);
+        for (int u = 0; u < kU; u++) v[u] = e + u * step < n4 ? __ldg(x4 + e + u * step) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int u = 0; u < 4; u++)
+        for (int u = 0; u < kU; u++)
           m32 = max(m32, max(max(v[u].x & 0x7FFFFFFFu, v[u].y & 0x7FFFFFFFu),
                              max(v[u].z & 0x7FFFFFFFu, v[u].w & 0x7FFFFFFFu)));
       }
-      for (int64_t e = (n4 << 2) + threadIdx.x; e < n; e += blockDim.x)
-        m32 = max(m32, __float_as_uint(__ldg(xf + e)) & 0x7FFFFFFFu);
+      for (int64_t e = (n4 << 2) + first; e < n; e += step) m32 = max(m32, __float_as_uint(__ldg(xf + e)) & 0x7FFFFFFFu);
     }
     // as a double's magnitude bits: equal exponent of the top bit, so exponent_above agrees
     if (m32 >= kInfBits32)
@@ -107,29 +134,39 @@ __global__ void __launch_bounds__(256) split_exp_kernel(SplitArgs a) {
     else if (m32)
       mx = (unsigned long long)(exponent_above32(m32) + 1022) << 52;
   } else if (off >= 0) {
-    // tiles start 16-byte aligned (even offsets): pairs of doubles, four pairs in flight
+    // tiles start 16-byte aligned (even offsets): pairs of doubles
     const longlong2* x2 = reinterpret_cast<const longlong2*>(x);
     const int64_t n2 = n >> 1;
-    const int64_t bd = blockDim.x;
-    for (int64_t e = threadIdx.x; e < n2; e += 4 * bd) {
-      longlong2 v[4];
+    for (int64_t e = first; e < n2; e += kU * step) {
+      longlong2 v[kU];
 #pragma unroll
-      for (int u = 0; u < 4; u++) v[u] = e + u * bd < n2 ? __ldg(x2 + e + u * bd) : make_longlong2(0, 0);
+      for (int u = 0; u < kU; u++) v[u] = e + u * step < n2 ? __ldg(x2 + e + u * step) : make_longlong2(0, 0);
 #pragma unroll
-      for (int u = 0; u < 4; u++) {
+      for (int u = 0; u < kU; u++) {
         mx = max(mx, (unsigned long long)v[u].x & kAbsMask);
         mx = max(mx, (unsigned long long)v[u].y & kAbsMask);
       }
     }
-    if ((n & 1) && threadIdx.x == 0) mx = max(mx, mag_bits(__ldg(x + n - 1)));
+    if ((n & 1) && first == 0) mx = max(mx, mag_bits(__ldg(x + n - 1)));
   }
-  __shared__ unsigned long long red[8];
+  __shared__ unsigned long long red[kExpThreads / 32];
+  __shared__ unsigned long long part[kExpCluster];
   for (int o = 16; o; o >>= 1) mx = max(mx, (unsigned long long)__shfl_xor_sync(0xffffffffu, (long long)mx, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
+  unsigned long long m = 0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < kExpThreads / 32; w++) m = max(m, red[w]);
+  if (nz > 1) {
+    cluster_wait();
+    if (threadIdx.x == 0) store_rank0(&part[z], m);
+    cluster_arrive();
+    cluster_wait();
+    if (z > 0) return;
+    if (threadIdx.x == 0)
+      for (int w = 0; w < nz; w++) m = max(m, part[w]);
+  }
   if (threadIdx.x == 0) {
-    unsigned long long m = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) m = max(m, red[w]);
     int e = 0;
     if (off < 0 || m >= kInfBits) {
       atomicOr(a.err, off < 0 ? kErrBadOffset : kErrNonFinite);
@@ -144,151 +181,137 @@ __global__ void __launch_bounds__(256) split_exp_kernel(SplitArgs a) {
 }
 
 // Row/column scaling: one exponent per row of each stored A tile and per column of each
-// stored B tile (kZeroLine for an all-zero line); a non-finite value is reported by
-// split_exp_kernel. One block per tile, one thread per line.
-__global__ void __launch_bounds__(256) split_exp_lines_kernel(SplitArgs a) {
+// stored B tile (kZeroLine for an all-zero line). One CTA per tile; a line whose elements are
+// contiguous is one warp's, lanes along it; otherwise lanes are neighbouring lines and the
+// warps share their elements, so loads are coalesced either way (a thread per line read the
+// contiguous ones 32 lines apart). Bound by HBM. Offsets and non-finite values are checked
+// here: the tile exponents are not needed.
+__global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_constant__ SplitArgs a) {
   const int b = blockIdx.x;
   const bool isA = b < a.n_a_tiles;
   const int t = isA ? a.a_tiles[b] : a.b_tiles[b - a.n_a_tiles];
   int rows, cols;
   int64_t off;
   tile_geometry(a, isA, t, rows, cols, off);
-  if (off < 0) return;
-  const double* x = (isA ? a.A : a.B) + off;
-  const int i_or_k = isA ? t / a.K : t / a.N;
-  const int k_or_j = isA ? t % a.K : t % a.N;
-  const int nl = isA ? rows : cols;   // lines
-  const int len = isA ? cols : rows;  // elements per line
-  const bool tr = isA ? a.transa != 0 : a.transb != 0;
-  // element u of line l: A row l is (l, u), B column l is (u, l); stored transposed or not
-  const int64_t lstep = isA ? (tr ? 1 : cols) : (tr ? rows : 1);
-  const int64_t ustep = isA ? (tr ? rows : 1) : (tr ? 1 : cols);
-  if (a.cplx) {
-    // complex elements: the plan's inner and column tilings count both parts, so an A tile
-    // is rows x (2 qc) and a B tile (2 qc) x (2 cc) of the real product; a line's exponent
-    // is that of the complex row (column) over both parts, and the B column cl and its
-    // partner cl + cc (the same complex column's other part) share it
-    const int qc = (isA ? cols : rows) >> 1;
-    const int nlc = isA ? rows : cols >> 1;  // complex lines
-    const int64_t cl_step = isA ? (tr ? 1 : qc) : (tr ? qc : 1);           // between lines
-    const int64_t cu_step = isA ? (tr ? rows : 1) : (tr ? 1 : (cols >> 1));  // along a line
-    const double* xc = (isA ? a.A : a.B) + 2 * off;
-    for (int l = threadIdx.x; l < nlc; l += blockDim.x) {
-      unsigned long long lm = 0;
-      const double* line = xc + 2 * (l * cl_step);
-      for (int u = 0; u < qc; u++) {
-        lm = max(lm, mag_bits(__ldg(line + 2 * u * cu_step)));
-        lm = max(lm, mag_bits(__ldg(line + 2 * u * cu_step + 1)));
-      }
-      const int e = (lm > 0 && lm < kInfBits) ? exponent_above(lm) : kZeroLine;
-      if (isA) {
-        a.eArow[(int64_t)k_or_j * a.Mtot + a.ro[i_or_k] + l] = e;
-      } else {
-        a.eBcol[(int64_t)i_or_k * a.Ntot + a.co[k_or_j] + l] = e;
-        a.eBcol[(int64_t)i_or_k * a.Ntot + a.co[k_or_j] + nlc + l] = e;
-      }
-    }
+  if (off < 0 || (a.f32 && (off & 3))) {
+    if (threadIdx.x == 0) atomicOr(a.err, kErrBadOffset);
     return;
   }
-  for (int l = threadIdx.x; l < nl; l += blockDim.x) {
+  const int i_or_k = isA ? t / a.K : t / a.N;
+  const int k_or_j = isA ? t % a.K : t % a.N;
+  const bool tr = isA ? a.transa != 0 : a.transb != 0;
+  // Complex elements: the plan's inner and column tilings count both parts, so an A tile is
+  // rows x (2 qc) and a B tile (2 qc) x (2 cc) of the real product; a line's exponent is that
+  // of the complex row (column) over both parts, and the B column c and its partner c + cc
+  // (the same complex column's other part) share it.
+  const int parts = a.cplx ? 2 : 1;
+  const int nl = isA ? rows : cols / parts;                 // lines
+  const int len = (isA ? cols : rows) / parts;              // elements (complex: pairs) per line
+  const bool contig = isA ? !tr : tr;
+  const double* const x = (isA ? a.A : a.B) + parts * off;
+  const float* const xf = (isA ? a.Af : a.Bf) + off;
+  int32_t* const out = isA ? a.eArow + (int64_t)k_or_j * a.Mtot + a.ro[i_or_k]
+                           : a.eBcol + (int64_t)i_or_k * a.Ntot + a.co[k_or_j];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // the largest magnitude's bits (a float's or a double's)
+  auto at = [&](int64_t e) -> unsigned long long {
+    return a.f32 ? (unsigned long long)(__float_as_uint(__ldg(xf + e)) & 0x7FFFFFFFu) : mag_bits(__ldg(x + e));
+  };
+  auto write = [&](int l, unsigned long long m) {
+    if (a.f32 ? m >= kInfBits32 : m >= kInfBits) atomicOr(a.err, kErrNonFinite);
     int e = kZeroLine;
     if (a.f32) {
-      uint32_t lm = 0;
-      const float* line = (isA ? a.Af : a.Bf) + off + l * lstep;
-      for (int u = 0; u < len; u++) lm = max(lm, __float_as_uint(__ldg(line + u * ustep)) & 0x7FFFFFFFu);
-      if (lm > 0 && lm < kInfBits32) e = exponent_above32(lm);
-    } else {
-      unsigned long long lm = 0;
-      const double* line = x + l * lstep;
-      for (int u = 0; u < len; u++) lm = max(lm, mag_bits(__ldg(line + u * ustep)));
-      if (lm > 0 && lm < kInfBits) e = exponent_above(lm);
+      if (m > 0 && m < kInfBits32) e = exponent_above32((uint32_t)m);
+    } else if (m > 0 && m < kInfBits) {
+      e = exponent_above(m);
     }
-    if (isA)
-      a.eArow[(int64_t)k_or_j * a.Mtot + a.ro[i_or_k] + l] = e;
-    else
-      a.eBcol[(int64_t)i_or_k * a.Ntot + a.co[k_or_j] + l] = e;
-  }
-}
-
-// ---------------------------------------------------------------- kernel 1b: largest exponents
-// Per row block i: Emax_A(i) = the largest exponent of its stored A tiles (0 when none);
-// the same per column block for B. One block per row or column block, its threads
-// spread over the K inner blocks. The contraction adds each tile pair's exact integer at
-// the binary position GUARD + rowexp + colexp of a 128-bit accumulator whose unit is
-// 2^(Emax_A(i) + Emax_B(j) - 7(s+1) - GUARD); the class kernel writes rowexp and colexp.
-__global__ void __launch_bounds__(256) split_emax_kernel(SplitArgs a) {
-  const bool isA = (int)blockIdx.x < a.M;
-  const int t = isA ? blockIdx.x : blockIdx.x - a.M;
-  int em = INT_MIN;
-  if (isA ? a.r[t] > 0 : a.c[t] > 0) {
-    for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
-      if (a.q[k] <= 0) continue;
-      if (isA) {
-        if (a.am[(int64_t)t * a.K + k]) em = max(em, a.eA[(int64_t)t * a.K + k]);
-      } else {
-        if (a.bm[(int64_t)k * a.N + t]) em = max(em, a.eB[(int64_t)k * a.N + t]);
+    out[l] = e;
+    if (!isA && a.cplx) out[nl + l] = e;
+  };
+  if (contig) {
+    const int n = len * parts;
+    for (int l = warp; l < nl; l += 8) {
+      unsigned long long m = 0;
+#pragma unroll 4
+      for (int u = lane; u < n; u += 32) m = max(m, at((int64_t)l * n + u));
+      for (int o = 16; o; o >>= 1) m = max(m, (unsigned long long)__shfl_xor_sync(0xffffffffu, (long long)m, o));
+      if (lane == 0) write(l, m);
+    }
+  } else {
+    __shared__ unsigned long long red[8][32];
+    for (int l0 = 0; l0 < nl; l0 += 32) {
+      const int l = l0 + lane;
+      unsigned long long m = 0;
+      if (l < nl) {
+#pragma unroll 4
+        for (int u = warp; u < len; u += 8) {
+          const int64_t e = ((int64_t)u * nl + l) * parts;
+          m = max(m, at(e));
+          if (parts == 2) m = max(m, at(e + 1));
+        }
       }
+      red[warp][lane] = m;
+      __syncthreads();
+      if (warp == 0 && l < nl) {
+        for (int w = 1; w < 8; w++) m = max(m, red[w][lane]);
+        write(l, m);
+      }
+      __syncthreads();
     }
-  }
-  __shared__ int red[8];
-  for (int o = 16; o; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = em;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++) em = max(em, red[w]);
-    if (em == INT_MIN) em = 0;
-    if (isA)
-      a.eAmax[t] = em;
-    else
-      a.eBmax[t] = em;
   }
 }
 
-// ---------------------------------------------------------------- kernel 1b': line scales
-// Row/column scaling: one thread per row m of A (per column n of B): Emax = the largest
-// exponent of that line over its stored tiles (all-zero lines excluded; 0 when none), and
-// rowexp[k][m] = e(m, k) - Emax (colexp likewise), 0 where there is no tile or the line is
-// zero there (its slices are zero).
-__global__ void __launch_bounds__(256) split_scale_lines_kernel(SplitArgs a) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < a.Mtot) {
-    const int64_t m = t;
-    const int i = a.row_tile[m];
-    int em = INT_MIN;
-    for (int k = 0; k < a.K; k++) {
-      const int e = a.eArow[(int64_t)k * a.Mtot + m];
-      if (a.am[(int64_t)i * a.K + k] && a.q[k] > 0 && e != kZeroLine) em = max(em, e);
+// ---------------------------------------------------------------- kernel 1b: line scales
+// Row/column scaling, per row m of A (per column n of B): Emax = the largest exponent of that
+// line over its stored tiles (all-zero lines excluded; 0 when none), and rowexp[k][m] =
+// e(m, k) - Emax (colexp likewise), 0 where there is no tile or the line is zero there (its
+// slices are zero). A CTA takes 32 lines, its warps the inner blocks in turn.
+__global__ void __launch_bounds__(256) split_scale_lines_kernel(const __grid_constant__ SplitArgs a) {
+  __shared__ int red[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t = (int64_t)blockIdx.x * 32 + lane;
+  const bool isA = t < a.Mtot;
+  const bool in = t < a.Mtot + a.Ntot;
+  const int64_t x = isA ? t : t - a.Mtot;
+  const int tile = in ? (isA ? a.row_tile[x] : a.col_tile[x]) : 0;
+  auto exponent = [&](int k) -> int {  // kZeroLine: no tile, or a zero line
+    if (a.q[k] <= 0 || !(isA ? a.am[(int64_t)tile * a.K + k] : a.bm[(int64_t)k * a.N + tile])) return kZeroLine;
+    return isA ? a.eArow[(int64_t)k * a.Mtot + x] : a.eBcol[(int64_t)k * a.Ntot + x];
+  };
+  int em = INT_MIN;
+  if (in) {
+#pragma unroll 4
+    for (int k = warp; k < a.K; k += 8) {
+      const int e = exponent(k);
+      if (e != kZeroLine) em = max(em, e);
     }
-    if (em == INT_MIN) em = 0;
-    a.eAmaxr[m] = em;
-    for (int k = 0; k < a.K; k++) {
-      const int e = a.eArow[(int64_t)k * a.Mtot + m];
-      const bool pres = a.am[(int64_t)i * a.K + k] && a.q[k] > 0 && e != kZeroLine;
-      a.rowexp[(int64_t)k * a.Mtot + m] = (int16_t)(pres ? e - em : 0);
-    }
-  } else if (t < a.Mtot + a.Ntot) {
-    const int64_t n = t - a.Mtot;
-    const int j = a.col_tile[n];
-    int em = INT_MIN;
-    for (int k = 0; k < a.K; k++) {
-      const int e = a.eBcol[(int64_t)k * a.Ntot + n];
-      if (a.bm[(int64_t)k * a.N + j] && a.q[k] > 0 && e != kZeroLine) em = max(em, e);
-    }
-    if (em == INT_MIN) em = 0;
-    a.eBmaxc[n] = em;
-    for (int k = 0; k < a.K; k++) {
-      const int e = a.eBcol[(int64_t)k * a.Ntot + n];
-      const bool pres = a.bm[(int64_t)k * a.N + j] && a.q[k] > 0 && e != kZeroLine;
-      a.colexp[(int64_t)k * a.colexp_ld + n] = (int16_t)(pres ? e - em : 0);
-    }
+  }
+  red[warp][lane] = em;
+  __syncthreads();
+  for (int w = 0; w < 8; w++) em = max(em, red[w][lane]);
+  if (em == INT_MIN) em = 0;
+  if (!in) return;
+  if (warp == 0) (isA ? a.eAmaxr : a.eBmaxc)[x] = em;
+#pragma unroll 4
+  for (int k = warp; k < a.K; k += 8) {
+    const int e = exponent(k);
+    const int16_t d = (int16_t)(e != kZeroLine ? e - em : 0);
+    if (isA)
+      a.rowexp[(int64_t)k * a.Mtot + x] = d;
+    else
+      a.colexp[(int64_t)k * a.colexp_ld + x] = d;
   }
 }
 
 // ---------------------------------------------------------------- kernel 1c: offsets and scale classes
-// One warp per (k block, row block) and per (k block, column block). With one scale per
-// tile it first writes the offsets of its rows, rowexp[k][m] = e_A(i,k) - Emax_A(i) for a
-// stored tile (0 for an absent one), or of its columns (colexp); with one scale per row
-// and column the line kernel wrote them.
+// For one block of lines (a 128-row block of A or a 32-column block of B) and a range of inner
+// blocks, by one CTA of the pack kernel's launch (slicing needs the exponents only, so it runs
+// beside this). With one scale per tile, first Emax of each of the block's tiles, the largest
+// exponent over all its stored tiles (0 when none), and then the offsets of the block's
+// lines, rowexp[k][m] = e_A(i,k) - Emax_A(i) for a stored tile (0 for an absent one), or
+// colexp; with one scale per row and column the line kernel wrote them. The contraction adds
+// each tile pair's exact integer at the binary position GUARD + rowexp + colexp of a 128-bit
+// accumulator whose unit is 2^(Emax_A + Emax_B - 7(s+1) - GUARD).
 // Then the scale class. The products of k block k land at element (m, n) at the binary
 // position e_A(m,k) + e_B(n,k) - Emax_A(m) - Emax_B(n) (exponents of the row's and the
 // column's tile, or line, at k, and their maxima). When the rows of the row block that
@@ -300,81 +323,114 @@ __global__ void __launch_bounds__(256) split_scale_lines_kernel(SplitArgs a) {
 // guard + urow + ucol + rowadj[m] + coladj[n]. kNonUniform marks a k block whose rows (or
 // columns) at k have different exponents; rows without a tile (or all-zero lines) there
 // take no part.
-__global__ void __launch_bounds__(256) split_class_kernel(SplitArgs a) {
-  // one warp per (k block, row block) and per (k block, column block); lanes over the lines
-  const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t nr = (int64_t)a.K * a.RB, nc = (int64_t)a.K * a.CB;
-  int lo = INT_MAX, hi = INT_MIN, emx = INT_MIN;
-  if (wid < nr) {
-    const int k = (int)(wid / a.RB), rb = (int)(wid % a.RB);
-    const int64_t m0 = (int64_t)rb * kSplitBM;
-    const int64_t m1 = m0 + kSplitBM < a.Mtot ? m0 + kSplitBM : a.Mtot;
-    for (int64_t m = m0 + lane; m < m1; m += 32) {
-      const int i = a.row_tile[m];
-      const int emax_m = a.rowscale ? a.eAmaxr[m] : a.eAmax[i];
-      emx = max(emx, emax_m);
-      bool pres = a.q[k] > 0 && a.am[(int64_t)i * a.K + k];
-      int eabs = 0;
+//
+// A CTA takes chains of a few dependent loads, so there are at most kClassMaxRanges of them
+// per block of lines, fewer where the blocks are many, and they stand between the slicing
+// CTAs of the launch, which use the memory meanwhile (all in front, and 16 per block, they
+// held the banded 32768 product's launch for 260 us).
+constexpr int kClassMaxRanges = 16;
+
+struct ClassShared {
+  int32_t tile[kSplitBM];  // the lines' tiles
+  int32_t em[kSplitBM];    // and largest exponents
+  uint32_t first[kSplitBM / 32];  // bit: the line is the first of its tile here
+};
+
+__device__ void scale_classes(const SplitArgs& a, ClassShared& sm, int item, int nr) {
+  const int blk = item / nr;
+  const bool isA = blk < a.RB;
+  const int b = isA ? blk : blk - a.RB;
+  const int k0 = (int)((int64_t)(item % nr) * a.K / nr), k1 = (int)((int64_t)(item % nr + 1) * a.K / nr);
+  const int width = isA ? kSplitBM : 32;
+  const int64_t x0 = (int64_t)b * width;
+  const int64_t total = isA ? a.Mtot : a.Ntot;
+  const int nl = (int)min((int64_t)width, total - x0);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < kSplitBM) {
+    int t = -1;
+    bool first = false;
+    if (tid < nl) {
+      const int32_t* const of = isA ? a.row_tile : a.col_tile;
+      t = of[x0 + tid];
+      first = tid == 0 || of[x0 + tid - 1] != t;
+      if (a.rowscale) sm.em[tid] = isA ? a.eAmaxr[x0 + tid] : a.eBmaxc[x0 + tid];
+    }
+    sm.tile[tid] = t;
+    const uint32_t bits = __ballot_sync(0xffffffffu, first);
+    if (lane == 0) sm.first[warp] = bits;
+  }
+  __syncthreads();
+  if (!a.rowscale) {
+    for (int l = warp; l < nl; l += 8) {
+      if (!(sm.first[l >> 5] >> (l & 31) & 1)) continue;
+      const int t = sm.tile[l];
+      int em = INT_MIN;
+#pragma unroll 4
+      for (int k = lane; k < a.K; k += 32) {
+        const int64_t at = isA ? (int64_t)t * a.K + k : (int64_t)k * a.N + t;
+        const int e = __ldg((isA ? a.eA : a.eB) + at);
+        if (__ldg(a.q + k) > 0 && __ldg((isA ? a.am : a.bm) + at)) em = max(em, e);
+      }
+      for (int o = 16; o; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+      if (lane == 0) sm.em[l] = em == INT_MIN ? 0 : em;
+    }
+    __syncthreads();
+    int em = 0;
+    if (tid < nl) {  // the line that is first in this line's tile
+      int w = tid >> 5;
+      uint32_t bits = sm.first[w] & (0xffffffffu >> (31 - (tid & 31)));
+      while (!bits) bits = sm.first[--w];
+      em = sm.em[w * 32 + 31 - __clz((int)bits)];
+    }
+    __syncthreads();
+    if (tid < nl) sm.em[tid] = em;
+    __syncthreads();
+  }
+  int emx = INT_MIN;
+  for (int l = lane; l < nl; l += 32) emx = max(emx, sm.em[l]);
+  for (int o = 16; o; o >>= 1) emx = max(emx, __shfl_xor_sync(0xffffffffu, emx, o));
+  if (k0 == 0 && tid < nl) {
+    (isA ? a.emaxr : a.emaxc)[x0 + tid] = sm.em[tid];
+    if (a.urow) (isA ? a.rowadj : a.coladj)[x0 + tid] = (int16_t)(emx - sm.em[tid]);
+  }
+  const uint8_t* const mask = isA ? a.am : a.bm;
+  const int32_t* const exps = isA ? a.eA : a.eB;
+#pragma unroll 4
+  for (int k = k0 + warp; k < k1; k += 8) {
+    const bool some = __ldg(a.q + k) > 0;
+    int lo = INT_MAX, hi = INT_MIN;
+#pragma unroll
+    for (int u = 0; u < kSplitBM / 32; u++) {
+      const int l = u * 32 + lane;
+      if (l >= nl) continue;
+      const int t = sm.tile[l];
+      const int64_t at = isA ? (int64_t)t * a.K + k : (int64_t)k * a.N + t;
+      bool pres = __ldg(mask + at) != 0 && some;
+      int e = 0;
       if (!a.rowscale) {
-        eabs = pres ? a.eA[(int64_t)i * a.K + k] : 0;
-        a.rowexp[(int64_t)k * a.Mtot + m] = (int16_t)(pres ? eabs - emax_m : 0);
+        const int ev = __ldg(exps + at);  // (whatever is there when no tile is stored)
+        e = pres ? ev : 0;
+        const int16_t d = (int16_t)(pres ? e - sm.em[l] : 0);
+        if (isA)
+          a.rowexp[(int64_t)k * a.Mtot + x0 + l] = d;
+        else
+          a.colexp[(int64_t)k * a.colexp_ld + x0 + l] = d;
       } else if (pres) {
-        eabs = a.eArow[(int64_t)k * a.Mtot + m];
-        pres = eabs != kZeroLine;
+        e = isA ? a.eArow[(int64_t)k * a.Mtot + x0 + l] : a.eBcol[(int64_t)k * a.Ntot + x0 + l];
+        pres = e != kZeroLine;
       }
       if (pres) {
-        lo = min(lo, eabs);
-        hi = max(hi, eabs);
+        lo = min(lo, e);
+        hi = max(hi, e);
       }
     }
     for (int o = 16; o; o >>= 1) {
       lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
       hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      emx = max(emx, __shfl_xor_sync(0xffffffffu, emx, o));
     }
-    if (k == 0)
-      for (int64_t m = m0 + lane; m < m1; m += 32) {
-        const int e = a.rowscale ? a.eAmaxr[m] : a.eAmax[a.row_tile[m]];
-        a.emaxr[m] = e;
-        if (a.urow) a.rowadj[m] = (int16_t)(emx - e);
-      }
-    if (a.urow && lane == 0) a.urow[wid] = (int16_t)(lo > hi ? 0 : lo == hi ? lo - emx : kNonUniform);
-  } else if (wid < nr + nc) {
-    const int64_t u = wid - nr;
-    const int k = (int)(u / a.CB), cb = (int)(u % a.CB);
-    const int64_t n0 = (int64_t)cb * a.tn;
-    const int64_t n1 = n0 + a.tn < a.Ntot ? n0 + a.tn : a.Ntot;
-    for (int64_t n = n0 + lane; n < n1; n += 32) {
-      const int j = a.col_tile[n];
-      const int emax_n = a.rowscale ? a.eBmaxc[n] : a.eBmax[j];
-      emx = max(emx, emax_n);
-      bool pres = a.q[k] > 0 && a.bm[(int64_t)k * a.N + j];
-      int eabs = 0;
-      if (!a.rowscale) {
-        eabs = pres ? a.eB[(int64_t)k * a.N + j] : 0;
-        a.colexp[(int64_t)k * a.colexp_ld + n] = (int16_t)(pres ? eabs - emax_n : 0);
-      } else if (pres) {
-        eabs = a.eBcol[(int64_t)k * a.Ntot + n];
-        pres = eabs != kZeroLine;
-      }
-      if (pres) {
-        lo = min(lo, eabs);
-        hi = max(hi, eabs);
-      }
-    }
-    for (int o = 16; o; o >>= 1) {
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      emx = max(emx, __shfl_xor_sync(0xffffffffu, emx, o));
-    }
-    if (k == 0)
-      for (int64_t n = n0 + lane; n < n1; n += 32) {
-        const int e = a.rowscale ? a.eBmaxc[n] : a.eBmax[a.col_tile[n]];
-        a.emaxc[n] = e;
-        if (a.ucol) a.coladj[n] = (int16_t)(emx - e);
-      }
-    if (a.ucol && lane == 0) a.ucol[u] = (int16_t)(lo > hi ? 0 : lo == hi ? lo - emx : kNonUniform);
+    int16_t* const cls = isA ? a.urow : a.ucol;
+    if (cls && lane == 0)
+      cls[isA ? (int64_t)k * a.RB + b : (int64_t)k * a.CB + b] = (int16_t)(lo > hi ? 0 : lo == hi ? lo - emx : kNonUniform);
   }
 }
 
@@ -649,14 +705,34 @@ struct PackEntry {
   int32_t pass0;  // its first pass
 };
 
+struct PackGrid {
+  int ncls, ranges, every;  // CTAs for the scale classes, per block of lines, and their spacing
+  int ny;                   // CTAs per group of lines to pack
+};
+
 template <typename T, int S, typename E, bool CPLX = false>
-__global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __grid_constant__ SplitArgs a, int ny) {
-  __shared__ PackLine lines[kPackLines];
-  __shared__ PackEntry entries[kPackEntries];
-  __shared__ int passes_of[kPackEntries];
+__global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __grid_constant__ SplitArgs a, PackGrid g) {
+  __shared__ union {
+    ClassShared cls;
+    struct {
+      PackLine lines[kPackLines];
+      PackEntry entries[kPackEntries];
+      int passes_of[kPackEntries];
+    } pk;
+  } sm;
+  const int turn = blockIdx.x / g.every;  // every g.every-th CTA: offsets and scale classes
+  if (turn < g.ncls && blockIdx.x % g.every == 0) {
+    scale_classes(a, sm.cls, turn, g.ranges);
+    return;
+  }
+  auto& lines = sm.pk.lines;
+  auto& entries = sm.pk.entries;
+  auto& passes_of = sm.pk.passes_of;
+  const int bid = blockIdx.x - min(g.ncls, turn + 1);
+  const int ny = g.ny;
   constexpr int VE = 16 / (int)sizeof(E);
   const int tid = threadIdx.x;
-  const int grp = blockIdx.x / ny;
+  const int grp = bid / ny;
   const bool isA = grp < a.n_a_blocks;
   const bool contig = isA ? !a.transa : a.transb != 0;  // a line's inner elements are contiguous
   if (tid < kPackLines) {
@@ -772,7 +848,7 @@ __global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __gri
         *reinterpret_cast<uint4*>(pc.dst + (size_t)t * slice_stride) = make_uint4(0u, 0u, 0u, 0u);
     }
   };
-  int pass = blockIdx.x % ny;
+  int pass = bid % ny;
   if (pass >= total) return;
   Piece cur, nxt;
   load(cur, pass);
@@ -789,63 +865,89 @@ __global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __gri
 }  // namespace
 
 template <typename E, bool C = false>
-cudaError_t launch_pack(const SplitArgs& a, cudaStream_t st) {
+cudaError_t launch_pack(const SplitArgs& a, PackGrid pg, cudaStream_t st) {
   // CTAs per group: one, or as many (up to a pass each) as fill the resident grid, where a
   // group's passes one after the other would be most of a small product's time
   const int groups = a.n_a_blocks + (a.n_b_blocks + kPackEntries - 1) / kPackEntries;
   const int passes = 2 * ((a.qmax + kSplitKC - 1) / kSplitKC);
   const int ny = std::max(1, std::min({kPackMaxY, passes, kPackResident / std::max(1, groups)}));
-  const unsigned g = (unsigned)(groups * ny);
+  const unsigned g = (unsigned)(pg.ncls + groups * ny);
+  if (g == 0) return cudaSuccess;
+  pg.ny = ny;
+  pg.every = std::max(1, pg.ncls ? (int)(g / pg.ncls) * 3 / 4 : 1);
   switch (a.s * 2 + (a.fp16 ? 1 : 0)) {
-    case 2: split_pack_kernel<__nv_bfloat16, 1, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 3: split_pack_kernel<__half, 1, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 4: split_pack_kernel<__nv_bfloat16, 2, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 5: split_pack_kernel<__half, 2, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 6: split_pack_kernel<__nv_bfloat16, 3, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 7: split_pack_kernel<__half, 3, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 8: split_pack_kernel<__nv_bfloat16, 4, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 9: split_pack_kernel<__half, 4, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 10: split_pack_kernel<__nv_bfloat16, 5, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 11: split_pack_kernel<__half, 5, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 12: split_pack_kernel<__nv_bfloat16, 6, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
-    case 13: split_pack_kernel<__half, 6, E, C><<<g, kPackThreads, 0, st>>>(a, ny); break;
+    case 2: split_pack_kernel<__nv_bfloat16, 1, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 3: split_pack_kernel<__half, 1, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 4: split_pack_kernel<__nv_bfloat16, 2, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 5: split_pack_kernel<__half, 2, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 6: split_pack_kernel<__nv_bfloat16, 3, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 7: split_pack_kernel<__half, 3, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 8: split_pack_kernel<__nv_bfloat16, 4, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 9: split_pack_kernel<__half, 4, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 10: split_pack_kernel<__nv_bfloat16, 5, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 11: split_pack_kernel<__half, 5, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 12: split_pack_kernel<__nv_bfloat16, 6, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 13: split_pack_kernel<__half, 6, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
+// CTAs of the pack launch that write offsets and scale classes: the blocks of lines, each in
+// as many ranges of inner blocks (of 8 at least) as make about two of a resident grid
+static PackGrid class_grid(const SplitArgs& a) {
+  PackGrid g{0, 1, 1, 1};
+  const int blocks = a.RB + a.CB;
+  if (!(a.urow || !a.rowscale) || a.K == 0 || blocks == 0) return g;
+  g.ranges = std::max(1, std::min({kClassMaxRanges, (a.K + 7) / 8, 2 * kPackResident / blocks}));
+  g.ncls = blocks * g.ranges;
+  return g;
+}
+
 int split_prep_kernels(const SplitArgs& a) {  // the kernels launch_split_prep launches
   int n = 0;
-  if (a.n_a_tiles + a.n_b_tiles > 0) n += a.rowscale ? 2 : 1;
-  if (a.rowscale ? a.Mtot + a.Ntot > 0 : a.M + a.N > 0) n++;
-  if ((a.urow || !a.rowscale) && (int64_t)a.K * (a.RB + a.CB) > 0) n++;
-  if (a.n_a_blocks + a.n_b_blocks > 0) n++;
+  if (a.n_a_tiles + a.n_b_tiles > 0) n++;
+  if (a.rowscale && a.Mtot + a.Ntot > 0) n++;
+  if (class_grid(a).ncls + a.n_a_blocks + a.n_b_blocks > 0) n++;
   return n;
 }
 
 cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* ev, int* k) {
-  if (a.n_a_tiles + a.n_b_tiles > 0) {
-    split_exp_kernel<<<a.n_a_tiles + a.n_b_tiles, 256, 0, st>>>(a);
-    if (a.rowscale) split_exp_lines_kernel<<<a.n_a_tiles + a.n_b_tiles, 256, 0, st>>>(a);
+  const int tiles = a.n_a_tiles + a.n_b_tiles;
+  if (tiles > 0 && a.rowscale) {
+    split_exp_lines_kernel<<<tiles, 256, 0, st>>>(a);
+  } else if (tiles > 0) {
+    int nz = 1;  // CTAs per tile: up to a resident grid's worth of CTAs in all
+    while (nz < kExpCluster && 2 * nz * tiles <= kExpResident) nz *= 2;
+    if (nz == 1) {
+      split_exp_kernel<<<tiles, kExpThreads, 0, st>>>(a);
+    } else {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(tiles * nz);
+      cfg.blockDim = dim3(kExpThreads);
+      cfg.stream = st;
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = nz;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      const cudaError_t e = cudaLaunchKernelEx(&cfg, split_exp_kernel, a);
+      if (e != cudaSuccess) return e;
+    }
   }
   if (a.rowscale) {
-    // the per-tile maxima (eAmax/eBmax) are not used in this mode; the line kernel writes
-    // rowexp/colexp and the line maxima
+    // the line maxima, and rowexp/colexp
     const int64_t lines = a.Mtot + a.Ntot;
-    if (lines > 0) split_scale_lines_kernel<<<(unsigned)((lines + 255) / 256), 256, 0, st>>>(a);
-  } else if (a.M + a.N > 0) {
-    split_emax_kernel<<<a.M + a.N, 256, 0, st>>>(a);
+    if (lines > 0) split_scale_lines_kernel<<<(unsigned)((lines + 31) / 32), 256, 0, st>>>(a);
   }
-  // tile scaling: the offsets rowexp/colexp; both: the scale classes (when kept)
-  const int64_t ncls = (int64_t)a.K * (a.RB + a.CB);
-  if ((a.urow || !a.rowscale) && ncls > 0) split_class_kernel<<<(unsigned)((ncls * 32 + 255) / 256), 256, 0, st>>>(a);
   if (ev) cudaEventRecord(ev[++*k], st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (a.n_a_blocks + a.n_b_blocks > 0) {
-    cudaError_t pe = a.f32 ? launch_pack<float>(a, st) : a.cplx ? launch_pack<double, true>(a, st) : launch_pack<double>(a, st);
-    if (pe != cudaSuccess) return pe;
-  }
+  const PackGrid pg = class_grid(a);
+  e = a.f32 ? launch_pack<float>(a, pg, st)
+            : a.cplx ? launch_pack<double, true>(a, pg, st) : launch_pack<double>(a, pg, st);
+  if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[++*k], st);
   return cudaGetLastError();
 }

@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const __grid_constant
   const int64_t m = (int64_t)rd.rb * kSplitBM + row;
   const bool row_ok = m < a.Mtot;
   const int Lrow =
-      row_ok ? (a.rowscale ? a.eAmaxr[m] : a.eAmax[a.row_tile[m]]) - kSplitBeta * (a.s + 1) - kSplitGuard : 0;
+      row_ok ? a.emaxr[m] - kSplitBeta * (a.s + 1) - kSplitGuard : 0;
   const int64_t n0 = (int64_t)cb * TN + warp * kCols;
   const size_t piece_stride = (size_t)a.cl * TN * kSplitBM;
   const uint4* src =
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const __grid_constant
     const int64_t n = n0 + c;
     unsigned long long v = 0ull;
     if (row_ok && n < a.Ntot) {
-      const int L = Lrow + (a.rowscale ? a.eBmaxc[n] : a.eBmax[a.col_tile[n]]);
+      const int L = Lrow + a.emaxc[n];
       v = a.f32 ? acc_bits_any<true>(w[c][0], w[c][1], w[c][2], w[c][3], L)
                 : acc_bits_any<false>(w[c][0], w[c][1], w[c][2], w[c][3], L);
     }
