@@ -173,6 +173,7 @@ std::vector<int32_t> choose_pieces(const std::vector<double>& cost, const std::v
   const double avg = total / std::max(1, bins);
   if (mx <= avg / kGran[sizeof(kGran) / sizeof(kGran[0]) - 1]) return one;  // no candidate cuts a unit
   double best = 0.9 * lpt_makespan(cost, one, bins, overhead);
+  if (best <= avg) return one;  // no packing is shorter than the bins' average load
   std::vector<int32_t> pick = one;
   for (int g : kGran) {
     const double target = avg / g;

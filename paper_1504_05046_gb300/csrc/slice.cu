@@ -181,11 +181,14 @@ __global__ void __launch_bounds__(kExpThreads) split_exp_kernel(const __grid_con
 }
 
 // Row/column scaling: one exponent per row of each stored A tile and per column of each
-// stored B tile (kZeroLine for an all-zero line). One CTA per tile; a line whose elements are
+// stored B tile (kZeroLine for an all-zero line). A few CTAs per tile; a line whose elements are
 // contiguous is one warp's, lanes along it; otherwise lanes are neighbouring lines and the
 // warps share their elements, so loads are coalesced either way (a thread per line read the
-// contiguous ones 32 lines apart). Bound by HBM. Offsets and non-finite values are checked
-// here: the tile exponents are not needed.
+// contiguous ones 32 lines apart), 8 of them in flight per thread. Bound by HBM: complex 3072
+// (302 MB), A transposed, 92 us; a CTA per tile with one load after the other 160 us. Offsets
+// and non-finite values are checked here: the tile exponents are not needed.
+constexpr int kLinesY = 4;  // CTAs per tile, sharing its lines
+template <typename E>
 __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_constant__ SplitArgs a) {
   const int b = blockIdx.x;
   const bool isA = b < a.n_a_tiles;
@@ -193,7 +196,7 @@ __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_const
   int rows, cols;
   int64_t off;
   tile_geometry(a, isA, t, rows, cols, off);
-  if (off < 0 || (a.f32 && (off & 3))) {
+  if (off < 0 || (std::is_same<E, float>::value && (off & 3))) {
     if (threadIdx.x == 0) atomicOr(a.err, kErrBadOffset);
     return;
   }
@@ -208,19 +211,23 @@ __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_const
   const int nl = isA ? rows : cols / parts;                 // lines
   const int len = (isA ? cols : rows) / parts;              // elements (complex: pairs) per line
   const bool contig = isA ? !tr : tr;
-  const double* const x = (isA ? a.A : a.B) + parts * off;
-  const float* const xf = (isA ? a.Af : a.Bf) + off;
+  constexpr bool kF32 = std::is_same<E, float>::value;
+  const E* const x = reinterpret_cast<const E*>(kF32 ? (const void*)(isA ? a.Af : a.Bf) : (const void*)(isA ? a.A : a.B)) +
+                     parts * off;
   int32_t* const out = isA ? a.eArow + (int64_t)k_or_j * a.Mtot + a.ro[i_or_k]
                            : a.eBcol + (int64_t)i_or_k * a.Ntot + a.co[k_or_j];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // the largest magnitude's bits (a float's or a double's)
   auto at = [&](int64_t e) -> unsigned long long {
-    return a.f32 ? (unsigned long long)(__float_as_uint(__ldg(xf + e)) & 0x7FFFFFFFu) : mag_bits(__ldg(x + e));
+    if constexpr (kF32)
+      return __float_as_uint(__ldg(x + e)) & 0x7FFFFFFFu;
+    else
+      return mag_bits(__ldg(x + e));
   };
   auto write = [&](int l, unsigned long long m) {
-    if (a.f32 ? m >= kInfBits32 : m >= kInfBits) atomicOr(a.err, kErrNonFinite);
+    if (kF32 ? m >= kInfBits32 : m >= kInfBits) atomicOr(a.err, kErrNonFinite);
     int e = kZeroLine;
-    if (a.f32) {
+    if constexpr (kF32) {
       if (m > 0 && m < kInfBits32) e = exponent_above32((uint32_t)m);
     } else if (m > 0 && m < kInfBits) {
       e = exponent_above(m);
@@ -230,24 +237,44 @@ __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_const
   };
   if (contig) {
     const int n = len * parts;
-    for (int l = warp; l < nl; l += 8) {
+    for (int l = warp + 8 * blockIdx.y; l < nl; l += 8 * kLinesY) {
       unsigned long long m = 0;
-#pragma unroll 4
-      for (int u = lane; u < n; u += 32) m = max(m, at((int64_t)l * n + u));
+      constexpr int kU = 8;  // loads in flight
+      for (int u0 = lane; u0 < n; u0 += 32 * kU) {
+        unsigned long long v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) v[u] = u0 + 32 * u < n ? at((int64_t)l * n + u0 + 32 * u) : 0ull;
+#pragma unroll
+        for (int u = 0; u < kU; u++) m = max(m, v[u]);
+      }
       for (int o = 16; o; o >>= 1) m = max(m, (unsigned long long)__shfl_xor_sync(0xffffffffu, (long long)m, o));
       if (lane == 0) write(l, m);
     }
   } else {
     __shared__ unsigned long long red[8][32];
-    for (int l0 = 0; l0 < nl; l0 += 32) {
+    for (int l0 = 32 * blockIdx.y; l0 < nl; l0 += 32 * kLinesY) {
       const int l = l0 + lane;
       unsigned long long m = 0;
       if (l < nl) {
-#pragma unroll 4
-        for (int u = warp; u < len; u += 8) {
-          const int64_t e = ((int64_t)u * nl + l) * parts;
-          m = max(m, at(e));
-          if (parts == 2) m = max(m, at(e + 1));
+        constexpr int kU = 8;  // loads in flight
+        for (int u0 = warp; u0 < len; u0 += 8 * kU) {
+          if (parts == 2) {  // both parts of a complex element at once (16-byte aligned)
+            longlong2 v[kU];
+#pragma unroll
+            for (int u = 0; u < kU; u++) {
+              const int64_t e = ((int64_t)(u0 + 8 * u) * nl + l) * 2;
+              v[u] = u0 + 8 * u < len ? __ldg(reinterpret_cast<const longlong2*>(x + e)) : make_longlong2(0, 0);
+            }
+#pragma unroll
+            for (int u = 0; u < kU; u++)
+              m = max(m, max((unsigned long long)v[u].x & kAbsMask, (unsigned long long)v[u].y & kAbsMask));
+          } else {
+            unsigned long long v[kU];
+#pragma unroll
+            for (int u = 0; u < kU; u++) v[u] = u0 + 8 * u < len ? at((int64_t)(u0 + 8 * u) * nl + l) : 0ull;
+#pragma unroll
+            for (int u = 0; u < kU; u++) m = max(m, v[u]);
+          }
         }
       }
       red[warp][lane] = m;
@@ -915,7 +942,10 @@ int split_prep_kernels(const SplitArgs& a) {  // the kernels launch_split_prep l
 cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* ev, int* k) {
   const int tiles = a.n_a_tiles + a.n_b_tiles;
   if (tiles > 0 && a.rowscale) {
-    split_exp_lines_kernel<<<tiles, 256, 0, st>>>(a);
+    if (a.f32)
+      split_exp_lines_kernel<float><<<dim3(tiles, kLinesY), 256, 0, st>>>(a);
+    else
+      split_exp_lines_kernel<double><<<dim3(tiles, kLinesY), 256, 0, st>>>(a);
   } else if (tiles > 0) {
     int nz = 1;  // CTAs per tile: up to a resident grid's worth of CTAs in all
     while (nz < kExpCluster && 2 * nz * tiles <= kExpResident) nz *= 2;
