@@ -81,7 +81,8 @@ __device__ __forceinline__ void wide_store(const SplitArgs& P, uint32_t (&acc)[T
   using E = std::conditional_t<ELEM == 1, float, double>;
   if (m0 >= P.Mtot || n0 >= P.Ntot) return;
   const E alpha = (E)P.alpha, beta = (E)P.beta;
-  const bool scale = __double_as_longlong(P.alpha) != __double_as_longlong(1.0);
+  const Factor fa(P.alpha), fb(P.beta);
+  const bool scale = !fa.one;
   const bool accum = (__double_as_longlong(P.beta) & 0x7FFFFFFFFFFFFFFFll) != 0;
   E* const C = reinterpret_cast<E*>(ELEM == 1 ? (void*)P.Cf : (void*)P.C);
   int it[4], lrow[4];  // the lane's rows m0 + 8 r + lane / 4: row tile (-1: none) and row in it
@@ -156,8 +157,8 @@ __device__ __forceinline__ void wide_store(const SplitArgs& P, uint32_t (&acc)[T
         if (accum) v = __fadd_rn(v, __fmul_rn(beta, old[r]));
       } else {
         v = __longlong_as_double((long long)x);
-        if (scale) v = __dmul_rn(alpha, v);
-        if (accum) v = __dadd_rn(v, __dmul_rn(beta, old[r]));
+        v = fa.times(v);
+        if (accum) v = __dadd_rn(v, fb.times(old[r]));
       }
       if (in && dst[r]) {
         *dst[r] = v;
