@@ -26,10 +26,11 @@ constexpr int kSplitMaxS = 6;      // slices per operand
 constexpr int kSplitEpiWarps = 8;  // epilogue warps (2 per TMEM lane quadrant)
 constexpr int kSplitGuard = 55;    // guard bits of the 128-bit accumulator below the largest scale
 constexpr double kEpiWalkBlocks = 32.0;  // mean k blocks per unit from which the epilogue walks
-// mean inner depth of a unit from which the 64-column form is taken: with many units per
-// group of CTAs, and always
-constexpr double kWideDepthMany = 2048.0, kWideDepth = 3072.0;
+// mean inner depth of a unit from which the 64-column form is taken: with packed pairs, with
+// many units per group of CTAs, and always
+constexpr double kWideDepthPairs = 1536.0, kWideDepthMany = 2048.0, kWideDepth = 3072.0;
 constexpr int64_t kWideManyUnits = 8;
+constexpr int kWidePairsMaxS = 4;  // slices up to which that form's column blocks are packed in pairs
 constexpr int kSplitMaxK = 8192;   // inner blocks per product
 constexpr int64_t kSplitMaxInner = int64_t(1) << 22;  // inner elements per product (128-bit sums' headroom)
 
@@ -129,8 +130,11 @@ struct SplitArgs {
   int32_t cl, CBG;          // CTAs per column-block group; groups (units are (rb, group))
   int32_t sw;               // the contraction kernel's form: 1 = with C store warps
   int32_t deep;             // 1: some inner block is deeper than kdepth (the kernel's DEEP form)
-  int32_t wide, wstages;    // 1: a plan of its own runs in the 64-column form (wide.cu) with this ring
-                            // depth; its groups are then of cl/2 CTAs, two column blocks each
+  // 1: a plan of its own runs in the 64-column form (wide.cu) with this ring depth; its groups
+  // are then of cl/2 CTAs, two column blocks each. pairs (3 and 4 slices): each pair of column
+  // blocks is packed slice by slice: a chunk of the pair holds, for every slice, block 2c's
+  // part and then block 2c+1's (bpk_off points at the block's own part of the first slice)
+  int32_t wide, wstages, pairs;
   int32_t epi_walk;         // 1: the epilogue finds the accumulation groups on its own k list
                             // (long lists); 0: it takes them from the MMA warps' descriptors
   int64_t Mtot, Ntot;
@@ -315,6 +319,7 @@ struct bsmm_plan_s {
   int epi_walk = 0;          // the epilogue walks the k lists itself (SplitArgs::epi_walk)
   int32_t qmax = 0;          // the largest inner block
   int wide = 0, wstages = 0; // the contraction runs in the 64-column form (SplitArgs::wide)
+  int pairs = 0;             // column blocks packed in pairs (SplitArgs::pairs)
   int deep = 0;              // some inner block is deeper than the exact FP32 depth
   int64_t Mtot = 0, Ntot = 0, colexp_ld = 0;
   int64_t apk_bytes = 0, bpk_bytes = 0;

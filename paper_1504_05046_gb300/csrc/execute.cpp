@@ -113,6 +113,7 @@ void fill_split_args(bsmm_plan_s* p, SplitArgs& a, double alpha, const void* A, 
   a.sw = p->sw;
   a.wide = p->wide;
   a.wstages = p->wstages;
+  a.pairs = p->pairs;
   a.epi_walk = p->epi_walk;
   a.deep = p->deep;
   a.f32 = p->opt.elem == BSMM_F32;

@@ -483,15 +483,9 @@ bsmm_status plan_split(bsmm_plan_s* p) {
         cur += (int64_t)log2i_ceil_div(p->q[k], kSplitKC) * a_chunk_bytes;
       }
   p->apk_bytes = cur;
-  cur = 0;
   for (int k = 0; k < K; k++)
     for (int cb = 0; cb < CB; cb++)
-      if (presB[(size_t)cb * KW + k / 64] >> (k % 64) & 1) {
-        bpk_off[(size_t)k * CB + cb] = cur;
-        b_blocks.push_back(k * CB + cb);
-        cur += (int64_t)log2i_ceil_div(p->q[k], kSplitKC) * b_chunk_bytes;
-      }
-  p->bpk_bytes = cur;
+      if (presB[(size_t)cb * KW + k / 64] >> (k % 64) & 1) b_blocks.push_back(k * CB + cb);
 
   // per C tile: sum over its k-list of 2*q_k (useful flops per element)
   std::vector<double> w((size_t)M * N, 0.0);
@@ -594,7 +588,11 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   //   6 slices, dense n = 2048: 290 / 324 us, 2560: 553 / 568, 3072: 970 / 888, 4096: 2214 /
   //   1979, 6144: 7188 / 6290, 16384: 133.1 / 112.3 ms; Bernoulli(0.5) masks, 8192 (2048 deep,
   //   54 units per group): 3970 / 3820; 512 x 32768 deep: 331 / 269
-  //   4 slices: 202 / 214, 375 / 363, 646 / 575, 1488 / 1296, 4953 / 4126; 2563 / 2337; 238 / 204
+  //   4 slices (packed in pairs), n = 1024: 39.1 / 41.1, 1280: 62.1 / 77.7, 1536: 94.7 / 86.5,
+  //   2048: 207 / 179, 4096: 1506 / 1015, 6144: 5168 / 3150; Bernoulli(0.5), 4096 (1024 deep):
+  //   356 / 370, 8192: 2651 / 2039; 512 x 131072 deep: 796 / 471
+  //   3 slices: 38.5 / 38.6, 60.8 / 71.4, 90.2 / 76.9, 193 / 150, 1398 / 820, 4764 / 2535;
+  //   355 / 350, 2622 / 1793; 736 / 370
   p->wide = 0;
   if (CL >= 2 && s >= 3 && p->sw && !p->deep && !base.empty()) {
     bool pairs = true;
@@ -604,10 +602,28 @@ bsmm_status plan_split(bsmm_plan_s* p) {
     for (int32_t k : bk) depth += p->q[k];
     depth /= (double)base.size();
     const bool many = (int64_t)base.size() >= kWideManyUnits * (p->sms / (CL / 2));
-    p->wide = pairs && depth >= (many ? kWideDepthMany : kWideDepth) ? 1 : 0;
+    p->wide = pairs && depth >= (s <= kWidePairsMaxS ? kWideDepthPairs : many ? kWideDepthMany : kWideDepth) ? 1 : 0;
     const int deepest = split_wide_stages(s);
     p->wstages = p->opt.stages ? std::min(p->opt.stages, deepest) : deepest;
   }
+  // where the column blocks' slices go: block by block, or pair by pair (SplitArgs::pairs; a
+  // last block without a partner leaves its partner's place empty)
+  p->pairs = p->wide && s <= kWidePairsMaxS;
+  cur = 0;
+  for (int32_t b : b_blocks) {
+    const int k = b / CB, cb = b % CB;
+    const int64_t bytes = (int64_t)log2i_ceil_div(p->q[k], kSplitKC) * b_chunk_bytes;
+    if (!p->pairs) {
+      bpk_off[b] = cur;
+      cur += bytes;
+    } else if (cb % 2 == 0) {
+      bpk_off[b] = cur;
+      cur += 2 * bytes;
+    } else {  // its partner has the same inner blocks and comes just before it
+      bpk_off[b] = bpk_off[b - 1] + b_chunk_bytes / s;
+    }
+  }
+  p->bpk_bytes = cur;
   const std::vector<int32_t> np =
       choose_pieces(bcost, blen, machine_bins(p), kSplitPieceOverhead, p->opt.ksplit == -1 ? 0 : p->opt.ksplit);
   std::vector<int32_t> slot0(base.size(), -1);

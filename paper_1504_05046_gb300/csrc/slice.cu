@@ -815,7 +815,9 @@ __global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __gri
 
   const E* const src = isA ? reinterpret_cast<const E*>(std::is_same<E, float>::value ? (const void*)a.Af : (const void*)a.A)
                            : reinterpret_cast<const E*>(std::is_same<E, float>::value ? (const void*)a.Bf : (const void*)a.B);
-  const int slice_stride = isA ? kSplitBM * kSplitKC * 2 : 32 * kSplitKC * 2;
+  // (a pair of column blocks packed together: the other block's part lies between the slices)
+  int slice_stride = isA ? kSplitBM * kSplitKC * 2 : 32 * kSplitKC * 2;
+  if constexpr (S <= kWidePairsMaxS) slice_stride <<= !isA && a.pairs;
   uint8_t* const pk = isA ? a.apk : a.bpk;
   const int ch = tid & 3;
 

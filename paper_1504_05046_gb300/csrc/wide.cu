@@ -18,7 +18,7 @@
 // first group runs.
 // Contraction, 32-column form against this one: dense 16384, 6 slices, 133.1 to 112.3 ms
 // (1645 TFLOP/s of slice products, 0.98 of what cuBLAS sustains in BF16); float32 8192, 4
-// slices, 11.68 to 9.67 ms; thin 512 x 524288 4.29 to 3.45 ms. The rule that takes it is the
+// slices, 11.68 to 7.64 ms; thin 512 x 524288 4.29 to 3.45 ms. The rule that takes it is the
 // planner's (plan.cpp).
 //
 // Roles: warp 0 producer, warps 1 and 2 MMA issue, warp 3 idle, warps 4 to 11 epilogue. The
@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
   constexpr int A_STAGE = S * kAChunk;
   constexpr int B_HALF = 32 * kSplitKC * 2;      // one slice of a 32-column block's chunk
   constexpr int B_STAGE = S * 2 * B_HALF;
+  constexpr bool PAIRS = S <= kWidePairsMaxS;    // column blocks packed in pairs
   constexpr int STAGE = A_STAGE + B_STAGE;
   constexpr int BUF_COLS = S * kWideN;
   constexpr int NB = 2 * BUF_COLS <= (int)kTmemCols ? 2 : 1;  // accumulator buffers
@@ -262,8 +263,12 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
     regs_dec<kWideRegsCtl>();
     if (warp == 0) {
       // ---------------------------------------------------------- producer
-      // The whole warp walks the list; per chunk lane 0 copies A and lanes 0..2S-1 one slice
-      // of one of the two column blocks each (interleaved into 64-row slices).
+      // The whole warp walks the list. With 3 and 4 slices a pair of column blocks is packed as
+      // it is read here, 64 rows per slice, and a chunk is two copies. From the 32-column
+      // packing it is 2S + 1, about 100 cycles each to issue: with 4 slices the tensor core
+      // waited for them a quarter of the time (float32 8192: 9.66 ms, 7.64 with two). With 5
+      // and 6 slices it does not: the dense 16384 product took 111.2 ms with 13 copies and
+      // 111.7 with two.
       int stage = 0;
       uint32_t phase = 0;
       uint32_t issued = 0, issued_par = 0;  // bit st: stage st holds an issued copy; its parity
@@ -271,24 +276,36 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
       for (int idx = ubeg; idx < uend && ok; idx++) {
         const SplitUnit un = a.units[a.sched_units[idx]];
         const int cb = un.cb * CL + 2 * rank;
-        const int cb1 = cb + 1 < a.CB ? cb + 1 : cb;  // a last, single block stands in for both
+        [[maybe_unused]] const int cb1 = cb + 1 < a.CB ? cb + 1 : cb;  // a last, single block stands in for both
         UnitIter it;
         it.init(a, un, cb);
         for (int kt = it.next_own(); kt >= 0 && ok; kt = it.next_own()) {
           const int nkc = (a.q[kt] + kSplitKC - 1) / kSplitKC;
           const uint8_t* asrc = a.apk + a.apk_off[(size_t)un.rb * a.K + kt];
-          const uint8_t* bsrc = a.bpk + a.bpk_off[(size_t)kt * a.CB + (lane & 1 ? cb1 : cb)] + (lane >> 1) * B_HALF;
+          const uint8_t* bsrc;
+          if constexpr (PAIRS)
+            bsrc = a.bpk + a.bpk_off[(size_t)kt * a.CB + cb];
+          else
+            bsrc = a.bpk + a.bpk_off[(size_t)kt * a.CB + (lane & 1 ? cb1 : cb)] + (lane >> 1) * B_HALF;
           for (int kc = 0; kc < nkc; kc++) {
             if (!wait_warp(&empty[stage], phase ^ 1, abort_flag, a.err)) {
               ok = false;
               break;
             }
             uint8_t* sa = smem + (size_t)stage * STAGE;
-            if (lane == 0) mbar_arrive_expect_tx(&full[stage], STAGE);
-            __syncwarp();
-            if (lane == 0) bulk_g2s(sa, asrc + (size_t)kc * A_STAGE, A_STAGE, &full[stage]);
-            if (lane < 2 * S)
-              bulk_g2s(sa + A_STAGE + lane * B_HALF, bsrc + (size_t)kc * (S * B_HALF), B_HALF, &full[stage]);
+            if constexpr (PAIRS) {
+              if (elect_one()) {
+                mbar_arrive_expect_tx(&full[stage], STAGE);
+                bulk_g2s(sa, asrc + (size_t)kc * A_STAGE, A_STAGE, &full[stage]);
+                bulk_g2s(sa + A_STAGE, bsrc + (size_t)kc * B_STAGE, B_STAGE, &full[stage]);
+              }
+            } else {  // lane l: slice l / 2 of block l % 2
+              if (lane == 0) mbar_arrive_expect_tx(&full[stage], STAGE);
+              __syncwarp();
+              if (lane == 0) bulk_g2s(sa, asrc + (size_t)kc * A_STAGE, A_STAGE, &full[stage]);
+              if (lane < 2 * S)
+                bulk_g2s(sa + A_STAGE + lane * B_HALF, bsrc + (size_t)kc * (S * B_HALF), B_HALF, &full[stage]);
+            }
             __syncwarp();
             issued |= 1u << stage;
             issued_par = (issued_par & ~(1u << stage)) | (phase << stage);

@@ -85,3 +85,32 @@ def test_pairs_that_differ_take_the_other_form():
     prob = G._assemble("pairs", r, c, q, am, bm, rng, "uniform", "pairs")
     _, plan, _ = check(prob, 6, cluster=2, ksplit=1)
     assert P.bsmm_plan_form(plan)["store_warps"] == 1
+
+
+@pytest.mark.parametrize("s", [3, 4, 6])
+def test_plans_of_the_form_in_a_batch(s):
+    """A batch runs every plan with the 32-column kernel: the same bits as each plan's own
+    execute, also with the column blocks packed in pairs (3 and 4 slices)."""
+    import torch
+    r, q, c = _sizes(15, 30, [40, 3, 90, 17])
+    probs = [_scaled_problem(20 + i, r, q, c, *CLASSES[k]) for i, k in enumerate(("one", "changes"))]
+    d = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    plans, args, alone = [], [], []
+    for p in probs:
+        plan = P.bsmm_plan(r, c, q, p.a_mask, p.b_mask, nslices=s, mode=P.BSMM_SPLIT_BF16, cluster=2, ksplit=1)
+        assert _is_wide(plan)
+        off, tot = G.layout_arena(P.bsmm_plan_query(plan)["c_mask"], r, c)
+        a = [d(p.A), d(p.a_off), d(p.B), d(p.b_off), torch.zeros(tot, dtype=torch.float64, device="cuda"), d(off)]
+        P.bsmm_execute(plan, 1.0, a[0], a[1], a[2], a[3], 0.0, a[4], a[5])
+        P.bsmm_status_device(plan)
+        alone.append(a[4].cpu().numpy())
+        a[4].zero_()
+        plans.append(plan)
+        args.append(a)
+    batch = P.bsmm_batch_create(plans)
+    P.bsmm_batch_set_args(batch, [1.0, 1.0], *[[a[i] for a in args] for i in range(4)], [0.0, 0.0],
+                          [a[4] for a in args], [a[5] for a in args])
+    P.bsmm_batch_execute(batch)
+    P.bsmm_batch_status_device(batch)
+    for a, want in zip(args, alone):
+        assert np.array_equal(a[4].cpu().numpy(), want)
