@@ -449,10 +449,12 @@ bsmm_status bsmm_batch_execute(bsmm_batch_t b, void* stream) {
           n++;
         }
     } else {
+      int last = 0;  // kernels of the last product's slicing
       for (int32_t i = b->wave_prod[w]; i < b->wave_prod[w + 1] && e == cudaSuccess; i++) {
         int k = 0;
         e = launch_split_prep(b->sargs[i], ws, nullptr, &k);
-        n += split_prep_kernels(b->sargs[i]);
+        last = split_prep_kernels(b->sargs[i]);
+        n += last;
       }
       if (e != cudaSuccess) break;
       SplitArgs a = b->sargs[0];
@@ -473,11 +475,11 @@ bsmm_status bsmm_batch_execute(bsmm_batch_t b, void* stream) {
       a.unit_prod = (const int32_t*)b->d_unit_prod.p;
       a.unit_local = (const int32_t*)b->d_unit_local.p;
       a.err = (int32_t*)b->d_err.p;
-      e = launch_split_mma(a, b->wave_bins[w], ws);
+      e = launch_split_mma(a, b->wave_bins[w], ws, last > 0);
       n++;
       for (int32_t i = b->wave_prod[w]; i < b->wave_prod[w + 1] && e == cudaSuccess; i++)
         if (b->sargs[i].n_red > 0) {
-          e = launch_split_reduce(b->sargs[i], ws);
+          e = launch_split_reduce(b->sargs[i], ws, true);
           n++;
         }
     }

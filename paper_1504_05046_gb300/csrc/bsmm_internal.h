@@ -232,18 +232,19 @@ struct SplitArgs {
 constexpr int kMaxEvents = 8;
 constexpr int kProfileRing = 64;  // executes whose per-kernel times a plan keeps
 cudaError_t launch_fp64(const Fp64Args& a, int ctas, cudaStream_t st, cudaEvent_t* ev, int* nk);
-cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEvent_t* ev, int* nk);
+// (after: the stream's previous operation is a kernel of the same call)
+cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEvent_t* ev, int* nk, bool after = false);
 // the two halves of launch_split: per-product exponents, scales and slices; the
 // persistent contraction over the schedule in `a` (clusters of a.cl CTAs)
-cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* ev, int* k);
+cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* ev, int* k, bool after = false);
 int split_prep_kernels(const SplitArgs& a);  // how many kernels launch_split_prep launches
-cudaError_t launch_split_mma(const SplitArgs& a, int clusters, cudaStream_t st);
+cudaError_t launch_split_mma(const SplitArgs& a, int clusters, cudaStream_t st, bool after);
 // the 64-column form (wide.cu): `groups` of a.cl/2 CTAs
-cudaError_t launch_split_wide(const SplitArgs& a, int groups, cudaStream_t st);
+cudaError_t launch_split_wide(const SplitArgs& a, int groups, cudaStream_t st, bool after);
 int split_wide_stages(int s);  // its deepest ring
 size_t split_wide_smem_bytes(int s, int stages);
 // split k: the reductions of the regions whose k-list was split (no launch when none)
-cudaError_t launch_split_reduce(const SplitArgs& a, cudaStream_t st);
+cudaError_t launch_split_reduce(const SplitArgs& a, cudaStream_t st, bool after);
 // a kernel whose bounded waits can never be satisfied (see bsmm_selftest_wait)
 cudaError_t launch_wait_selftest(int32_t* err, int64_t limit_ns, cudaStream_t st);
 cudaError_t launch_fp64_reduce(const Fp64Args& a, cudaStream_t st);

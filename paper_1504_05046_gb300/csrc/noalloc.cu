@@ -228,7 +228,7 @@ extern "C" bsmm_status bsmm_split_tile_noalloc(int32_t m, int32_t n, int32_t k, 
   a.part = nullptr;  // no split k: one inner block
   a.red = nullptr;
   a.n_red = 0;
-  e = launch_split(a, RB * CB, st, nullptr, nullptr);
+  e = launch_split(a, RB * CB, st, nullptr, nullptr, true);
   if (e != cudaSuccess) return set_error(std::string("noalloc launch: ") + cudaGetErrorString(e)), BSMM_ERR_CUDA;
   // the device error word, read back from the array itself (no buffer of the caller's)
   int32_t w = 0;

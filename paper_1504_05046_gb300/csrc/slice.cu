@@ -11,6 +11,7 @@
 #include <type_traits>
 
 #include "bsmm_internal.h"
+#include "overlap.cuh"
 
 namespace bsmm {
 
@@ -91,6 +92,7 @@ constexpr int kExpThreads = 256;
 constexpr int kExpCluster = 8;  // CTAs of a cluster, at most
 constexpr int kExpResident = 4 * 152;  // CTAs that fill the machine
 __global__ void __launch_bounds__(kExpThreads) split_exp_kernel(const __grid_constant__ SplitArgs a) {
+  grid_wait();
   const int nz = (int)cluster_size(), z = (int)cluster_rank();
   if (nz > 1) cluster_arrive();  // (waited for before rank 0's shared memory is written: it has started)
   const int b = blockIdx.x / nz;
@@ -190,6 +192,7 @@ __global__ void __launch_bounds__(kExpThreads) split_exp_kernel(const __grid_con
 constexpr int kLinesY = 4;  // CTAs per tile, sharing its lines
 template <typename E>
 __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_constant__ SplitArgs a) {
+  grid_wait();
   const int b = blockIdx.x;
   const bool isA = b < a.n_a_tiles;
   const int t = isA ? a.a_tiles[b] : a.b_tiles[b - a.n_a_tiles];
@@ -295,6 +298,7 @@ __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_const
 // slices are zero). A CTA takes 32 lines, its warps the inner blocks in turn.
 __global__ void __launch_bounds__(256) split_scale_lines_kernel(const __grid_constant__ SplitArgs a) {
   __shared__ int red[8][32];
+  grid_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t t = (int64_t)blockIdx.x * 32 + lane;
   const bool isA = t < a.Mtot;
@@ -747,6 +751,7 @@ __global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __gri
       int passes_of[kPackEntries];
     } pk;
   } sm;
+  grid_wait();
   const int turn = blockIdx.x / g.every;  // every g.every-th CTA: offsets and scale classes
   if (turn < g.ncls && blockIdx.x % g.every == 0) {
     scale_classes(a, sm.cls, turn, g.ranges);
@@ -894,7 +899,7 @@ __global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __gri
 }  // namespace
 
 template <typename E, bool C = false>
-cudaError_t launch_pack(const SplitArgs& a, PackGrid pg, cudaStream_t st) {
+cudaError_t launch_pack(const SplitArgs& a, PackGrid pg, cudaStream_t st, bool after) {
   // CTAs per group: one, or as many (up to a pass each) as fill the resident grid, where a
   // group's passes one after the other would be most of a small product's time
   const int groups = a.n_a_blocks + (a.n_b_blocks + kPackEntries - 1) / kPackEntries;
@@ -904,22 +909,24 @@ cudaError_t launch_pack(const SplitArgs& a, PackGrid pg, cudaStream_t st) {
   if (g == 0) return cudaSuccess;
   pg.ny = ny;
   pg.every = std::max(1, pg.ncls ? (int)(g / pg.ncls) * 3 / 4 : 1);
+  auto launch = [&](void (*kernel)(SplitArgs, PackGrid)) {
+    return launch_kernel(after, kernel, dim3(g), kPackThreads, 0, st, 1, a, pg);
+  };
   switch (a.s * 2 + (a.fp16 ? 1 : 0)) {
-    case 2: split_pack_kernel<__nv_bfloat16, 1, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 3: split_pack_kernel<__half, 1, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 4: split_pack_kernel<__nv_bfloat16, 2, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 5: split_pack_kernel<__half, 2, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 6: split_pack_kernel<__nv_bfloat16, 3, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 7: split_pack_kernel<__half, 3, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 8: split_pack_kernel<__nv_bfloat16, 4, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 9: split_pack_kernel<__half, 4, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 10: split_pack_kernel<__nv_bfloat16, 5, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 11: split_pack_kernel<__half, 5, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 12: split_pack_kernel<__nv_bfloat16, 6, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
-    case 13: split_pack_kernel<__half, 6, E, C><<<g, kPackThreads, 0, st>>>(a, pg); break;
+    case 2: return launch(split_pack_kernel<__nv_bfloat16, 1, E, C>);
+    case 3: return launch(split_pack_kernel<__half, 1, E, C>);
+    case 4: return launch(split_pack_kernel<__nv_bfloat16, 2, E, C>);
+    case 5: return launch(split_pack_kernel<__half, 2, E, C>);
+    case 6: return launch(split_pack_kernel<__nv_bfloat16, 3, E, C>);
+    case 7: return launch(split_pack_kernel<__half, 3, E, C>);
+    case 8: return launch(split_pack_kernel<__nv_bfloat16, 4, E, C>);
+    case 9: return launch(split_pack_kernel<__half, 4, E, C>);
+    case 10: return launch(split_pack_kernel<__nv_bfloat16, 5, E, C>);
+    case 11: return launch(split_pack_kernel<__half, 5, E, C>);
+    case 12: return launch(split_pack_kernel<__nv_bfloat16, 6, E, C>);
+    case 13: return launch(split_pack_kernel<__half, 6, E, C>);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 // CTAs of the pack launch that write offsets and scale classes: the blocks of lines, each in
@@ -941,44 +948,30 @@ int split_prep_kernels(const SplitArgs& a) {  // the kernels launch_split_prep l
   return n;
 }
 
-cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* ev, int* k) {
+cudaError_t launch_split_prep(const SplitArgs& a, cudaStream_t st, cudaEvent_t* ev, int* k, bool after) {
   const int tiles = a.n_a_tiles + a.n_b_tiles;
+  cudaError_t e = cudaSuccess;
   if (tiles > 0 && a.rowscale) {
-    if (a.f32)
-      split_exp_lines_kernel<float><<<dim3(tiles, kLinesY), 256, 0, st>>>(a);
-    else
-      split_exp_lines_kernel<double><<<dim3(tiles, kLinesY), 256, 0, st>>>(a);
+    const dim3 grid(tiles, kLinesY);
+    e = a.f32 ? launch_kernel(after, split_exp_lines_kernel<float>, grid, 256, 0, st, 1, a)
+              : launch_kernel(after, split_exp_lines_kernel<double>, grid, 256, 0, st, 1, a);
+    after = true;
   } else if (tiles > 0) {
     int nz = 1;  // CTAs per tile: up to a resident grid's worth of CTAs in all
     while (nz < kExpCluster && 2 * nz * tiles <= kExpResident) nz *= 2;
-    if (nz == 1) {
-      split_exp_kernel<<<tiles, kExpThreads, 0, st>>>(a);
-    } else {
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(tiles * nz);
-      cfg.blockDim = dim3(kExpThreads);
-      cfg.stream = st;
-      cudaLaunchAttribute at{};
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = nz;
-      at.val.clusterDim.y = at.val.clusterDim.z = 1;
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, split_exp_kernel, a);
-      if (e != cudaSuccess) return e;
-    }
+    e = launch_kernel(after, split_exp_kernel, dim3(tiles * nz), kExpThreads, 0, st, nz, a);
+    after = true;
   }
-  if (a.rowscale) {
-    // the line maxima, and rowexp/colexp
-    const int64_t lines = a.Mtot + a.Ntot;
-    if (lines > 0) split_scale_lines_kernel<<<(unsigned)((lines + 31) / 32), 256, 0, st>>>(a);
+  if (e != cudaSuccess) return e;
+  if (a.rowscale && a.Mtot + a.Ntot > 0) {  // the line maxima, and rowexp/colexp
+    e = launch_kernel(after, split_scale_lines_kernel, dim3((unsigned)((a.Mtot + a.Ntot + 31) / 32)), 256, 0, st, 1, a);
+    after = true;
   }
-  if (ev) cudaEventRecord(ev[++*k], st);
-  cudaError_t e = cudaGetLastError();
+  if (ev) cudaEventRecord(ev[++*k], st), after = false;
   if (e != cudaSuccess) return e;
   const PackGrid pg = class_grid(a);
-  e = a.f32 ? launch_pack<float>(a, pg, st)
-            : a.cplx ? launch_pack<double, true>(a, pg, st) : launch_pack<double>(a, pg, st);
+  e = a.f32 ? launch_pack<float>(a, pg, st, after)
+            : a.cplx ? launch_pack<double, true>(a, pg, st, after) : launch_pack<double>(a, pg, st, after);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[++*k], st);
   return cudaGetLastError();

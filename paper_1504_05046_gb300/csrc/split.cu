@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
+  grid_wait();  // the slices and classes; until here only the plan's own tables were read
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -598,6 +599,7 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const __grid_constant
   constexpr int kCols = TN * kRedRows / 256;  // columns per thread
   constexpr int kParts = kSplitBM / kRedRows;
   __shared__ unsigned long long cstage[kRedRows * (TN + 1)];
+  grid_wait();
   const int unit = blockIdx.x / kParts, part = blockIdx.x % kParts;
   const SplitRed rd = a.red[unit / a.cl];
   const int rank = unit % a.cl;
@@ -663,7 +665,7 @@ __global__ void __launch_bounds__(96) wait_selftest_kernel(int32_t* err, int64_t
 }
 
 template <int S, int TN, bool SW, bool WALK, bool DEEP = false>
-cudaError_t launch_mma(const SplitArgs& a, int groups, cudaStream_t st) {
+cudaError_t launch_mma(const SplitArgs& a, int groups, cudaStream_t st, bool after) {
   const size_t smem = split_smem_bytes(S, TN, a.stages);
   cudaError_t e = cudaFuncSetAttribute(split_mma_kernel<S, TN, SW, WALK, DEEP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -676,24 +678,24 @@ cudaError_t launch_mma(const SplitArgs& a, int groups, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     if (fa.numRegs != kRegsLaunch) return cudaErrorInvalidConfiguration;
   }
-  split_mma_kernel<S, TN, SW, WALK, DEEP><<<(unsigned)(groups * a.cl), threads_of<SW>(), smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(after, split_mma_kernel<S, TN, SW, WALK, DEEP>, dim3(groups * a.cl), threads_of<SW>(), smem, st, 1,
+                       a);
 }
 
 template <int S>
-cudaError_t launch_mma_sw(const SplitArgs& a, int groups, cudaStream_t st) {
+cudaError_t launch_mma_sw(const SplitArgs& a, int groups, cudaStream_t st, bool after) {
   if (a.cl != 1 && a.cl != 2 && a.cl != 4) return cudaErrorInvalidValue;
   // the walking epilogue is built for the forms with store warps and 3 to 6 slices (the
   // dense products' default); other forms take the descriptors whatever epi_walk says
   if (a.deep) {  // products with inner blocks deeper than the exact depth: store-warp forms
     if (!a.sw) return cudaErrorInvalidConfiguration;
     if constexpr (S >= 3)
-      if (a.epi_walk) return launch_mma<S, 32, true, true, true>(a, groups, st);
-    return launch_mma<S, 32, true, false, true>(a, groups, st);
+      if (a.epi_walk) return launch_mma<S, 32, true, true, true>(a, groups, st, after);
+    return launch_mma<S, 32, true, false, true>(a, groups, st, after);
   }
   if constexpr (S >= 3)
-    if (a.sw && a.epi_walk) return launch_mma<S, 32, true, true>(a, groups, st);
-  return a.sw ? launch_mma<S, 32, true, false>(a, groups, st) : launch_mma<S, 32, false, false>(a, groups, st);
+    if (a.sw && a.epi_walk) return launch_mma<S, 32, true, true>(a, groups, st, after);
+  return a.sw ? launch_mma<S, 32, true, false>(a, groups, st, after) : launch_mma<S, 32, false, false>(a, groups, st, after);
 }
 
 // Groups of cl CTAs that are resident at once: the persistent grid (one CTA per SM at
@@ -721,20 +723,21 @@ int max_groups_s(int cl, int stages, bool sw) {
 }  // namespace
 
 // NVTX ranges name the phases of a product for a timeline tool (host-side enqueue spans).
-cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEvent_t* ev, int* nk) {
+cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEvent_t* ev, int* nk, bool after) {
   int k = 0;
   if (ev) cudaEventRecord(ev[0], st);
   nvtxRangePushA("bsmm split: exponents, scales, slices");
-  cudaError_t e = launch_split_prep(a, st, ev, &k);
+  cudaError_t e = launch_split_prep(a, st, ev, &k, after);
   nvtxRangePop();
   if (e != cudaSuccess) return e;
   nvtxRangePushA("bsmm split: contraction");
-  e = a.wide && !a.prods ? launch_split_wide(a, ctas, st) : launch_split_mma(a, ctas, st);
+  after = !ev && split_prep_kernels(a) > 0;
+  e = a.wide && !a.prods ? launch_split_wide(a, ctas, st, after) : launch_split_mma(a, ctas, st, after);
   nvtxRangePop();
   if (ev) cudaEventRecord(ev[++k], st);
   if (e == cudaSuccess && !a.prods && a.n_red > 0) {  // a batch launches its products' reductions
     nvtxRangePushA("bsmm split: split-k reduction");
-    e = launch_split_reduce(a, st);
+    e = launch_split_reduce(a, st, !ev);
     nvtxRangePop();
     if (ev) cudaEventRecord(ev[++k], st);
   }
@@ -747,21 +750,20 @@ cudaError_t launch_wait_selftest(int32_t* err, int64_t limit_ns, cudaStream_t st
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_reduce(const SplitArgs& a, cudaStream_t st) {
+cudaError_t launch_split_reduce(const SplitArgs& a, cudaStream_t st, bool after) {
   if (a.n_red <= 0) return cudaSuccess;
-  split_reduce_kernel<32><<<(unsigned)(a.n_red * a.cl * (kSplitBM / kRedRows)), 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(after, split_reduce_kernel<32>, dim3(a.n_red * a.cl * (kSplitBM / kRedRows)), 256, 0, st, 1, a);
 }
 
-cudaError_t launch_split_mma(const SplitArgs& a, int ctas, cudaStream_t st) {
+cudaError_t launch_split_mma(const SplitArgs& a, int ctas, cudaStream_t st, bool after) {
   cudaError_t e;
   switch (a.s) {  // `ctas` counts groups of a.cl CTAs
-    case 1: e = launch_mma_sw<1>(a, ctas, st); break;
-    case 2: e = launch_mma_sw<2>(a, ctas, st); break;
-    case 3: e = launch_mma_sw<3>(a, ctas, st); break;
-    case 4: e = launch_mma_sw<4>(a, ctas, st); break;
-    case 5: e = launch_mma_sw<5>(a, ctas, st); break;
-    case 6: e = launch_mma_sw<6>(a, ctas, st); break;
+    case 1: e = launch_mma_sw<1>(a, ctas, st, after); break;
+    case 2: e = launch_mma_sw<2>(a, ctas, st, after); break;
+    case 3: e = launch_mma_sw<3>(a, ctas, st, after); break;
+    case 4: e = launch_mma_sw<4>(a, ctas, st, after); break;
+    case 5: e = launch_mma_sw<5>(a, ctas, st, after); break;
+    case 6: e = launch_mma_sw<6>(a, ctas, st, after); break;
     default: e = cudaErrorInvalidValue;
   }
   return e;

@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "bsmm_internal.h"
+#include "overlap.cuh"
 
 namespace bsmm {
 

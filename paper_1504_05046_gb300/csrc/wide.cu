@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
+  grid_wait();  // the slices and classes; until here only the plan's own tables were read
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -604,7 +605,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
 }
 
 template <int S>
-cudaError_t launch_wide(const SplitArgs& a, int groups, cudaStream_t st) {
+cudaError_t launch_wide(const SplitArgs& a, int groups, cudaStream_t st, bool after) {
   const size_t smem = split_wide_smem_bytes(S, a.wstages);
   cudaError_t e = cudaFuncSetAttribute(split_mma_wide_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -614,8 +615,7 @@ cudaError_t launch_wide(const SplitArgs& a, int groups, cudaStream_t st) {
   e = cudaFuncGetAttributes(&fa, split_mma_wide_kernel<S>);
   if (e != cudaSuccess) return e;
   if (fa.numRegs != kWideRegsLaunch) return cudaErrorInvalidConfiguration;
-  split_mma_wide_kernel<S><<<(unsigned)(groups * (a.cl / 2)), kWideThreads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(after, split_mma_wide_kernel<S>, dim3(groups * (a.cl / 2)), kWideThreads, smem, st, 1, a);
 }
 
 }  // namespace
@@ -631,13 +631,13 @@ int split_wide_stages(int s) {
   return st;
 }
 
-cudaError_t launch_split_wide(const SplitArgs& a, int groups, cudaStream_t st) {
+cudaError_t launch_split_wide(const SplitArgs& a, int groups, cudaStream_t st, bool after) {
   if (a.cl != 2 && a.cl != 4) return cudaErrorInvalidValue;
   switch (a.s) {
-    case 3: return launch_wide<3>(a, groups, st);
-    case 4: return launch_wide<4>(a, groups, st);
-    case 5: return launch_wide<5>(a, groups, st);
-    case 6: return launch_wide<6>(a, groups, st);
+    case 3: return launch_wide<3>(a, groups, st, after);
+    case 4: return launch_wide<4>(a, groups, st, after);
+    case 5: return launch_wide<5>(a, groups, st, after);
+    case 6: return launch_wide<6>(a, groups, st, after);
     default: return cudaErrorInvalidValue;
   }
 }
