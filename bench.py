@@ -180,6 +180,13 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
+def contraction_kernel(form):
+    """The contraction kernel of a plan's launch form: the 64-column one has no store warps
+    and an epilogue that walks the k lists."""
+    wide = form["cluster"] >= 2 and form["store_warps"] == 0 and form["epi_walk"] == 1
+    return "split_mma_wide_kernel" if wide else "split_mma_kernel"
+
+
 def profiled_traffic():
     """DRAM bytes per launch of the contraction kernel from the committed ncu summary,
     valid only while the kernel source is unchanged since the capture."""
@@ -599,7 +606,7 @@ def run_single(args, rank, world):
     fp64 = {"value": tf(ms64), "ms_per_step": ms64, "kernel_ms": k64}
     pair = s * (s + 1) / 2 * F
     if head_split:
-        roof = {"bound": "tensor", "kernel": "split_mma_kernel", "achieved": pair / (k_split[cis] * 1e-3) / 1e12,
+        roof = {"bound": "tensor", "kernel": contraction_kernel(P.bsmm_plan_form(plan)), "achieved": pair / (k_split[cis] * 1e-3) / 1e12,
                 "peak": pk["bf16_tflops_sustained"], "unit": "TFLOP/s", "traffic": None,
                 "peak_source": f"{pk_src} bf16_tflops_sustained (MEASURED_PEAKS.json)",
                 "launch": P.bsmm_plan_form(plan)}
@@ -800,15 +807,16 @@ def run_dense(args, rank, world, local):
 
     # per-kernel live times (CUDA events on the launching stream)
     kk = np.array(kms)
-    k_names = ["split_exp_scale_class_kernels", "split_pack_kernel", "split_mma_kernel"]
+    contraction = contraction_kernel(P.bsmm_plan_form(plan))
+    k_names = ["split_exp_kernel", "split_pack_kernel", contraction]
     k_avg = {nm: float(kk[:, i].mean()) for i, nm in enumerate(k_names)}
-    t_mma = k_avg["split_mma_kernel"] * 1e-3
+    t_mma = k_avg[contraction] * 1e-3
     pk, pk_src = peaks()
     pair_flops = s * (s + 1) / 2 * F
     mma_tflops = pair_flops / t_mma / 1e12
     peak_tc = pk["bf16_tflops_sustained"]
     traffic = profiled_traffic()
-    roofline = {"bound": "tensor", "kernel": "split_mma_kernel", "achieved": mma_tflops, "peak": peak_tc,
+    roofline = {"bound": "tensor", "kernel": contraction, "achieved": mma_tflops, "peak": peak_tc,
                 "unit": "TFLOP/s", "frac": mma_tflops / peak_tc, "traffic": traffic,
                 "peak_source": f"{pk_src} bf16_tflops_sustained (MEASURED_PEAKS.json)",
                 "achieved_def": f"{s * (s + 1) // 2} slice-pair products x useful flops per launch / mean launch time",

@@ -17,14 +17,16 @@
 //
 // Kernels, in launch order (1 and 2 in slice.cu, the others here):
 //   1. split_exp_kernel   per stored tile: the exponent e (integer max reduction);
-//      split_emax_kernel  per row / column block: the largest tile exponent;
-//      split_class_kernel per (k block, row block / column block): the per-row /
-//                         per-column offsets from it and the scale classes.
+//                         with one scale per line, split_exp_lines_kernel and
+//                         split_scale_lines_kernel in its place.
 //   2. split_pack_kernel  per (128-row block, k block) of A and (k block, tn-column
 //                         block) of B: the s slices, stored as bf16/fp16 in the
 //                         exact shared-memory image the tensor core reads (K-major,
 //                         64-byte swizzle, 32-element chunks), so the contraction
-//                         kernel moves them with plain 1-D bulk copies.
+//                         kernel moves them with plain 1-D bulk copies. The same
+//                         launch writes, per (k block, row block / column block), the
+//                         per-row / per-column offsets from the block's largest
+//                         exponent and the scale classes.
 //   3. split_mma_kernel   persistent, one CTA per SM, warp-specialised:
 //                         warp 0 streams packed chunks into an S-stage shared-memory
 //                         ring with cp.async.bulk (several k panels in flight -- the
@@ -34,6 +36,8 @@
 //                         accumulators; warps 4..11 drain TMEM (zeroing it behind
 //                         them), recombine in integer arithmetic and store
 //                         C = alpha*fl(sum) + beta*C.
+//                         split_mma_wide_kernel (wide.cu) in its place for products of
+//                         long k lists.
 //   4. split_reduce_kernel only for a plan that cut k-lists (split k, Sec. 3.2, Fig. 2):
 //                         adds each cut region's exact partial sums and stores C.
 // A work unit is a 128-row x tn-column block of the global C index space over its
