@@ -573,8 +573,17 @@ __device__ __forceinline__ U tie_to_even(U V) {
   return low ? ((V & (low << 1)) ? V + 1 : V - 1) : V;
 }
 
-// The window of one element, subnormals and tiny tiles included (r: the shift may be a left
-// one). Out of line: only tiles whose largest element is below 2^-900 need it.
+// Largest exponent e of a tile (line) in which an element with exponent field 0, which
+// decode<false> takes for a normal one, may leave bits in its window: it is then taken for a
+// value below 2^-1022 (a float for one below 2^-126), and its V for one below
+// 2^(-1022 + 7S + 2 - e), so above this e it is 0.
+template <int S, typename E>
+constexpr int kAnyExponent = 7 * S + 3 - (std::is_same<E, float>::value ? 128 : 1024);
+
+// The window of one element, subnormals and tiny tiles included (the shift may be a left
+// one). Out of line: only tiles of exponent kAnyExponent and below need it, for doubles
+// those of elements below 2^-979 or less, for floats below 2^-83 with six slices, 2^-97 with
+// four. (One bound of -900 for both types took a float's zero for 2^-127 there.)
 template <int S, typename E>
 __device__ __noinline__ unsigned long long slice_window_any(E x, int e) {
   uint32_t lo, hi, sgn;
@@ -594,7 +603,8 @@ __device__ __forceinline__ void slice_windows(const E (&x)[8], int e, uint32_t (
   // A normal element of a tile with max|x| < 2^e has be <= e + 1022, so V = m >> sh with
   // sh >= 51 - 7S. The significand's low kPre = 50 - 7S bits are below every V and with 4
   // slices or fewer are dropped first: what is left fits 32 bits. A zero or subnormal
-  // element's be = 0 shifts everything out: V = 0, as it should be.
+  // element (exponent field 0) shifts everything out: V = 0, as it should be, in tiles above
+  // kAnyExponent.
   constexpr int kPre = 50 - 7 * S;
   constexpr bool k32 = S <= 4;
   const int c = e + 1073 - 7 * S;
@@ -624,7 +634,7 @@ __device__ __forceinline__ void slice_windows(const E (&x)[8], int e, uint32_t (
       some = min(some, shl32(lo, 31 - sh));
     }
   }
-  if (e <= -900) {
+  if (e <= kAnyExponent<S, E>) {
 #pragma unroll
     for (int u = 0; u < 8; u++) {
       const unsigned long long V = slice_window_any<S>(x[u], e);
