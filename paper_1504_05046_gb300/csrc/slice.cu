@@ -63,7 +63,7 @@ constexpr uint32_t kInfBits32 = 0x7F800000u;
 __device__ __forceinline__ int exponent_above32(uint32_t m) {
   const int be = (int)(m >> 23);
   if (be) return be - 126;
-  return -126 - (__clz((int)m) - 8);  // subnormal: leading one at bit 31 - clz
+  return -126 - (__clz((int)m) - 9);  // subnormal: leading one at bit 31 - clz (22: below 2^-126)
 }
 
 __device__ __forceinline__ uint32_t cluster_size() {

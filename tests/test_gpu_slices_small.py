@@ -37,6 +37,14 @@ def test_small_tiles(shift, s):
         run_f32(_small(100, shift, False, False), s, mode)
 
 
+@pytest.mark.parametrize("s", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("shift", [-125, -126, -127, -133, -140, -147, -148])
+def test_tiles_of_subnormals(shift, s):
+    """Tiles (lines) whose largest element is subnormal: its exponent is that of its leading one."""
+    run_f32(_small(shift, 100, s % 2 == 1, True), s)
+    run_f32(_small(100, shift, False, False), s, scaling="rows")
+
+
 @pytest.mark.parametrize("s", [3, 6])
 @pytest.mark.parametrize("shift", [-950, -978, -979, -980, -999, -1000, -1001, -1040])
 def test_small_float64_tiles(shift, s):
