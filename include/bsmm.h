@@ -560,6 +560,15 @@ bsmm_status bsmm_status_device(bsmm_plan_t plan, void* stream);
 bsmm_status bsmm_selftest_wait(int64_t limit_ns, void* stream);
 
 /*
+ * The same for the grid barriers of bsmm_mlp_fit: fits a small model of its own with a barrier
+ * that waits limit_ns nanoseconds (1e6 .. 1e9) for one more arrival than there are CTAs, with
+ * (with_loss != 0) or without the final loss, and returns what bsmm_mlp_fit returned for it:
+ * BSMM_ERR_TIMEOUT, the device and the context staying usable. BSMM_ERR_INVALID for a limit
+ * out of range.
+ */
+bsmm_status bsmm_selftest_fit(int64_t limit_ns, int32_t with_loss, void* stream);
+
+/*
  * Per-unit timing records of the last execute with record_timings set:
  * start_ns[n_units], end_ns[n_units] (device %globaltimer, host outputs, either
  * may be NULL) and the CTA each unit ran on (cta[n_units], may be NULL). A split-mode

@@ -24,7 +24,7 @@ __all__ = [
     "bsmm_options_default", "bsmm_plan", "bsmm_plan_query", "bsmm_plan_ksplit", "bsmm_plan_features",
     "bsmm_plan_set_costs", "bsmm_plan_set_ctas", "bsmm_execute", "bsmm_execute_f32", "bsmm_execute_host",
     "bsmm_execute_host_async", "bsmm_host_wait", "bsmm_status_device", "BSMM_F64", "BSMM_F32", "BSMM_C128",
-    "bsmm_plan_timings", "bsmm_plan_kernel_ms", "bsmm_split_tile_noalloc", "bsmm_selftest_wait", "bsmm_last_error",
+    "bsmm_plan_timings", "bsmm_plan_kernel_ms", "bsmm_split_tile_noalloc", "bsmm_selftest_wait", "bsmm_selftest_fit", "bsmm_last_error",
     "bsmm_measure_rates", "bsmm_plan_form",
     "bsmm_destroy", "EXPORTED",
 ]
@@ -46,7 +46,7 @@ EXPORTED = [
     "bsmm_batch_execute", "bsmm_batch_query", "bsmm_batch_kernels", "bsmm_batch_set_costs", "bsmm_batch_status_device",
     "bsmm_batch_destroy", "bsmm_tune_space", "bsmm_batch_autotune", "bsmm_mlp_create", "bsmm_mlp_num_params", "bsmm_mlp_set_params", "bsmm_mlp_get_params",
     "bsmm_mlp_set_norm", "bsmm_mlp_get_norm", "bsmm_mlp_loss_grad", "bsmm_mlp_fit", "bsmm_mlp_predict",
-    "bsmm_plan_predict_costs", "bsmm_mlp_destroy", "bsmm_selftest_wait", "bsmm_schedule_lpt",
+    "bsmm_plan_predict_costs", "bsmm_mlp_destroy", "bsmm_selftest_wait", "bsmm_selftest_fit", "bsmm_schedule_lpt",
     "bsmm_schedule_pieces", "bsmm_measure_rates", "bsmm_mlp_save", "bsmm_mlp_load", "bsmm_plan_cost_source",
     "bsmm_execute_batch", "bsmm_batch_autotune_cached", "bsmm_plan_form", "bsmm_last_error", "bsmm_destroy",
 ]
@@ -105,6 +105,7 @@ def lib():
         L.bsmm_batch_query.argtypes = [P, P, P, P]
         L.bsmm_batch_kernels.argtypes = [P, P]
         L.bsmm_selftest_wait.argtypes = [i64, P]
+        L.bsmm_selftest_fit.argtypes = [i64, i32, P]
         L.bsmm_schedule_lpt.argtypes = [i64, P, i32, P, P, P]
         L.bsmm_schedule_pieces.argtypes = [i64, P, P, i32, f64, i32, P]
         L.bsmm_batch_set_costs.argtypes = [P, P]
@@ -444,6 +445,12 @@ def bsmm_selftest_wait(limit_ns: int, stream=None):
     """Runs the bounded-wait self-test kernel; raises BsmmError with status BSMM_ERR_TIMEOUT
     (4) when its waits ran out as designed."""
     _check(lib().bsmm_selftest_wait(int(limit_ns), _stream(stream)))
+
+
+def bsmm_selftest_fit(limit_ns: int, with_loss: bool = True, stream=None):
+    """Trains a small model whose grid barriers cannot complete; raises BsmmError with status
+    BSMM_ERR_TIMEOUT (4) when the training reported it as designed."""
+    _check(lib().bsmm_selftest_fit(int(limit_ns), int(with_loss), _stream(stream)))
 
 
 def bsmm_batch_kernels(batch: Batch) -> int:

@@ -112,9 +112,23 @@ __device__ __forceinline__ int64_t now_ns() {
   return (int64_t)t;
 }
 
-// Every CTA of the (cooperative) grid arrives; false when the wait ran out. `count` only
-// grows, by gridDim.x per barrier; sync[1] is the error flag.
-__device__ bool grid_barrier(unsigned* sync, unsigned target) {
+// A grid barrier's words: sync[0] counts arrivals (it only grows, by gridDim.x per barrier),
+// sync[1] is the error flag. `missing` is 0, or an arrival that the self-test waits for in
+// vain.
+struct Barrier {
+  unsigned* sync;
+  unsigned missing;
+  int64_t limit_ns;
+};
+
+// Every CTA of the (cooperative) grid arrives; false when the wait ran out, here or in
+// another CTA. One thread reads the flag for all: read by each of them, it could change in
+// between, and a part of the CTA would leave the kernel while the rest went on to the next
+// step's barriers.
+__device__ bool grid_barrier(const Barrier& b, unsigned arrivals) {
+  unsigned* const sync = b.sync;
+  const unsigned target = arrivals + b.missing;
+  bool ok = true;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -123,15 +137,15 @@ __device__ bool grid_barrier(unsigned* sync, unsigned target) {
     unsigned spin = 0;
     while ((int)(*(volatile unsigned*)&sync[0] - target) < 0) {  // (the count may wrap)
       if (*(volatile unsigned*)&sync[1]) break;
-      if ((++spin & 1023u) == 0 && now_ns() - t0 > kBarrierNs) {
+      if ((++spin & 1023u) == 0 && now_ns() - t0 > b.limit_ns) {
         atomicExch(&sync[1], 1u);
         break;
       }
     }
     __threadfence();
+    ok = *(volatile unsigned*)&sync[1] == 0u;
   }
-  __syncthreads();
-  return *(volatile unsigned*)&sync[1] == 0u;
+  return __syncthreads_and(ok);
 }
 
 // Sums over the tile's samples, in sample order: g[j][i] = sum a[q][j0 + j] b[q][i0 + i]
@@ -325,7 +339,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(float* para
                                                                   float* part, const __grid_constant__ Norm nm,
                                                                   const float* __restrict__ X,
                                                                   const float* __restrict__ t, int64_t n, int tiles,
-                                                                  int total, int updates, float lr, unsigned* sync) {
+                                                                  int total, int updates, float lr, Barrier bar) {
   extern __shared__ __align__(16) unsigned char raw[];
   TrainShared& sm = *reinterpret_cast<TrainShared*>(raw);
   const int tid = threadIdx.x, G = gridDim.x;
@@ -350,7 +364,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(float* para
     const bool keep = tiles <= kKeep * G;
     for (int tile = blockIdx.x, k = 0; tile < tiles; tile += G, k++)
       train_tile(sm, nm, X, t, n, tile, keep ? k : 0, keep && it > 0, part + (int64_t)tile * (NP + 1));
-    if (!grid_barrier(sync, (unsigned)(2 * it + 1) * G)) return;
+    if (!grid_barrier(bar, (unsigned)(2 * it + 1) * G)) return;
     // sums over the tiles in tile order: the CTA fetches a batch of its parameters' partial
     // sums at once, then a thread per parameter adds them
     const bool update = it < updates;
@@ -403,7 +417,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(float* para
         }
       }
     }
-    if (it + 1 < total && !grid_barrier(sync, (unsigned)(2 * it + 2) * G)) return;
+    if (it + 1 < total && !grid_barrier(bar, (unsigned)(2 * it + 2) * G)) return;
   }
 }
 
@@ -451,7 +465,7 @@ bsmm_status mlp_alloc(DevBuf& b, size_t bytes) {
 // mlp_train_kernel). The grid's CTAs wait for one another, so the launch is cooperative and
 // no larger than what is resident at once.
 bsmm_status train(bsmm_mlp_s* mlp, const float* X, const float* t, int64_t n, int total, int updates, float lr,
-                  cudaStream_t st) {
+                  cudaStream_t st, unsigned missing = 0, int64_t limit_ns = kBarrierNs) {
   const int64_t tiles64 = (n + TILE - 1) / TILE;
   if (tiles64 > (1 << 30)) return set_error("too many samples"), BSMM_ERR_INVALID;
   int tiles = (int)tiles64;
@@ -469,8 +483,8 @@ bsmm_status train(bsmm_mlp_s* mlp, const float* X, const float* t, int64_t n, in
     const int grid = std::max(1, std::min(tiles, sms * std::max(1, per_sm)));
     float *params = (float*)mlp->params.p, *m = (float*)mlp->m.p, *v = (float*)mlp->v.p, *grad = (float*)mlp->grad.p;
     float* part = (float*)mlp->part.p;
-    unsigned* sync = (unsigned*)mlp->sync.p;
-    void* args[] = {&params, &m, &v, &grad, &part, &mlp->norm, &X, &t, &n, &tiles, &total, &updates, &lr, &sync};
+    Barrier bar{(unsigned*)mlp->sync.p, missing, limit_ns};
+    void* args[] = {&params, &m, &v, &grad, &part, &mlp->norm, &X, &t, &n, &tiles, &total, &updates, &lr, &bar};
     e = cudaLaunchCooperativeKernel((const void*)mlp_train_kernel, dim3(grid), dim3(kTrainThreads), args,
                                     sizeof(TrainShared), st);
   }
@@ -481,6 +495,59 @@ bsmm_status train(bsmm_mlp_s* mlp, const float* X, const float* t, int64_t n, in
 // After a copy of the launch's outputs has been waited for: did a grid barrier run out?
 bsmm_status barrier_status(unsigned flag) {
   if (flag) return set_error("mlp training: a grid barrier timed out"), BSMM_ERR_TIMEOUT;
+  return BSMM_OK;
+}
+
+// bsmm_mlp_fit (`missing` and `limit_ns`: see Barrier)
+bsmm_status fit(bsmm_mlp_s* mlp, const float* X, const float* t, int64_t n, int32_t steps, float lr,
+                float* final_loss, void* stream, unsigned missing, int64_t limit_ns) {
+  if (!mlp || !X || !t || n <= 0 || steps < 0 || !(lr > 0.0f)) return set_error("bad arguments"), BSMM_ERR_INVALID;
+  cudaStream_t st = (cudaStream_t)stream;
+  // standardisation from the data (host, FP64 sums in sample order)
+  std::vector<float> hx((size_t)n * F), ht(n);
+  if (cudaMemcpyAsync(hx.data(), X, sizeof(float) * hx.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaMemcpyAsync(ht.data(), t, sizeof(float) * ht.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return set_error("copy failed"), BSMM_ERR_CUDA;
+  {
+    // (the features side by side: their sums are independent chains, each in sample order)
+    double s1[F] = {}, s2[F] = {}, mu[F];
+    for (int64_t i = 0; i < n; i++)
+      for (int f = 0; f < F; f++) s1[f] += hx[i * F + f];
+    for (int f = 0; f < F; f++) mu[f] = s1[f] / n;
+    for (int64_t i = 0; i < n; i++)
+      for (int f = 0; f < F; f++) s2[f] += (hx[i * F + f] - mu[f]) * (hx[i * F + f] - mu[f]);
+    for (int f = 0; f < F; f++) {
+      const double sd = std::sqrt(s2[f] / n);
+      mlp->norm.xmu[f] = (float)mu[f];
+      mlp->norm.xsd[f] = sd > 0 ? (float)sd : 1.0f;
+    }
+  }
+  {
+    double s1 = 0, s2 = 0;
+    for (int64_t i = 0; i < n; i++) s1 += ht[i];
+    const double mu = s1 / n;
+    for (int64_t i = 0; i < n; i++) s2 += (ht[i] - mu) * (ht[i] - mu);
+    const double sd = std::sqrt(s2 / n);
+    mlp->norm.ymu = (float)mu;
+    mlp->norm.ysd = sd > 0 ? (float)sd : 1.0f;
+  }
+  if (cudaMemsetAsync(mlp->m.p, 0, sizeof(float) * NP, st) != cudaSuccess ||
+      cudaMemsetAsync(mlp->v.p, 0, sizeof(float) * NP, st) != cudaSuccess)
+    return set_error("memset failed"), BSMM_ERR_CUDA;
+  const int total = steps + (final_loss ? 1 : 0);
+  if (total > 0) {
+    bsmm_status s = train(mlp, X, t, n, total, steps, lr, st, missing, limit_ns);
+    if (s != BSMM_OK) return s;
+  }
+  if (final_loss) {
+    unsigned flag = 0;
+    if (cudaMemcpyAsync(final_loss, (float*)mlp->grad.p + NP, sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&flag, (unsigned*)mlp->sync.p + 1, sizeof(flag), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+      return set_error("copy failed"), BSMM_ERR_CUDA;
+    return barrier_status(flag);
+  }
   return BSMM_OK;
 }
 
@@ -583,54 +650,24 @@ bsmm_status bsmm_mlp_loss_grad(bsmm_mlp_t mlp, const float* X, const float* t, i
 
 bsmm_status bsmm_mlp_fit(bsmm_mlp_t mlp, const float* X, const float* t, int64_t n, int32_t steps, float lr,
                          float* final_loss, void* stream) {
-  if (!mlp || !X || !t || n <= 0 || steps < 0 || !(lr > 0.0f)) return set_error("bad arguments"), BSMM_ERR_INVALID;
-  cudaStream_t st = (cudaStream_t)stream;
-  // standardisation from the data (host, FP64 sums in sample order)
-  std::vector<float> hx((size_t)n * F), ht(n);
-  if (cudaMemcpyAsync(hx.data(), X, sizeof(float) * hx.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaMemcpyAsync(ht.data(), t, sizeof(float) * ht.size(), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return set_error("copy failed"), BSMM_ERR_CUDA;
-  {
-    // (the features side by side: their sums are independent chains, each in sample order)
-    double s1[F] = {}, s2[F] = {}, mu[F];
-    for (int64_t i = 0; i < n; i++)
-      for (int f = 0; f < F; f++) s1[f] += hx[i * F + f];
-    for (int f = 0; f < F; f++) mu[f] = s1[f] / n;
-    for (int64_t i = 0; i < n; i++)
-      for (int f = 0; f < F; f++) s2[f] += (hx[i * F + f] - mu[f]) * (hx[i * F + f] - mu[f]);
-    for (int f = 0; f < F; f++) {
-      const double sd = std::sqrt(s2[f] / n);
-      mlp->norm.xmu[f] = (float)mu[f];
-      mlp->norm.xsd[f] = sd > 0 ? (float)sd : 1.0f;
-    }
-  }
-  {
-    double s1 = 0, s2 = 0;
-    for (int64_t i = 0; i < n; i++) s1 += ht[i];
-    const double mu = s1 / n;
-    for (int64_t i = 0; i < n; i++) s2 += (ht[i] - mu) * (ht[i] - mu);
-    const double sd = std::sqrt(s2 / n);
-    mlp->norm.ymu = (float)mu;
-    mlp->norm.ysd = sd > 0 ? (float)sd : 1.0f;
-  }
-  if (cudaMemsetAsync(mlp->m.p, 0, sizeof(float) * NP, st) != cudaSuccess ||
-      cudaMemsetAsync(mlp->v.p, 0, sizeof(float) * NP, st) != cudaSuccess)
-    return set_error("memset failed"), BSMM_ERR_CUDA;
-  const int total = steps + (final_loss ? 1 : 0);
-  if (total > 0) {
-    bsmm_status s = train(mlp, X, t, n, total, steps, lr, st);
-    if (s != BSMM_OK) return s;
-  }
-  if (final_loss) {
-    unsigned flag = 0;
-    if (cudaMemcpyAsync(final_loss, (float*)mlp->grad.p + NP, sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&flag, (unsigned*)mlp->sync.p + 1, sizeof(flag), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return set_error("copy failed"), BSMM_ERR_CUDA;
-    return barrier_status(flag);
-  }
-  return BSMM_OK;
+  return fit(mlp, X, t, n, steps, lr, final_loss, stream, 0, kBarrierNs);
+}
+
+bsmm_status bsmm_selftest_fit(int64_t limit_ns, int32_t with_loss, void* stream) {
+  if (limit_ns < 1000000 || limit_ns > 1000000000) return set_error("limit_ns must be in 1e6..1e9"), BSMM_ERR_INVALID;
+  constexpr int64_t n = 3 * TILE;  // three CTAs
+  bsmm_mlp_t mlp = nullptr;
+  DevBuf d;  // X, then t: all zero
+  bsmm_status s = bsmm_mlp_create(&mlp, 1);
+  if (s == BSMM_OK) s = mlp_alloc(d, sizeof(float) * n * (F + 1));
+  if (s == BSMM_OK && cudaMemsetAsync(d.p, 0, sizeof(float) * n * (F + 1), (cudaStream_t)stream) != cudaSuccess)
+    s = (set_error("memset failed"), BSMM_ERR_CUDA);
+  float loss = 0.0f;
+  const float* const X = (const float*)d.p;
+  if (s == BSMM_OK) s = fit(mlp, X, X + n * F, n, 2, 1e-3f, with_loss ? &loss : nullptr, stream, 1, limit_ns);
+  bsmm_mlp_destroy(mlp);  // (freeing waits for the kernel)
+  if (d.p) cudaFree(d.p);
+  return s;
 }
 
 bsmm_status bsmm_mlp_predict(bsmm_mlp_t mlp, const float* X, int64_t n, float* y, void* stream) {
