@@ -490,7 +490,9 @@ bsmm_status bsmm_batch_autotune_cached(bsmm_batch_t batch, const char* cache_pat
  * bsmm_mlp_fit         sets the standardisation from (X, t), then `steps` full-batch Adam
  *                      steps (beta1 0.9, beta2 0.999, eps 1e-8) at rate `lr`; reductions
  *                      run in a fixed order, so training is reproducible bit for bit;
- *                      *final_loss (host, may be NULL) after the last step
+ *                      *final_loss (host, may be NULL) after the last step; synchronises
+ *                      `stream`, and BSMM_ERR_TIMEOUT when a wait between the training
+ *                      kernel's CTAs ran out (the parameters are then those of some step)
  * bsmm_mlp_predict     y[n] device = predicted log time for X (device), asynchronous
  * bsmm_plan_predict_costs  predicts every unit of `plan` and re-packs it with the
  *                      predicted times as costs (bsmm_plan_set_costs); synchronises

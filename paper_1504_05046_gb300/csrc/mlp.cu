@@ -536,19 +536,17 @@ bsmm_status fit(bsmm_mlp_s* mlp, const float* X, const float* t, int64_t n, int3
       cudaMemsetAsync(mlp->v.p, 0, sizeof(float) * NP, st) != cudaSuccess)
     return set_error("memset failed"), BSMM_ERR_CUDA;
   const int total = steps + (final_loss ? 1 : 0);
-  if (total > 0) {
-    bsmm_status s = train(mlp, X, t, n, total, steps, lr, st, missing, limit_ns);
-    if (s != BSMM_OK) return s;
-  }
-  if (final_loss) {
-    unsigned flag = 0;
-    if (cudaMemcpyAsync(final_loss, (float*)mlp->grad.p + NP, sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&flag, (unsigned*)mlp->sync.p + 1, sizeof(flag), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return set_error("copy failed"), BSMM_ERR_CUDA;
-    return barrier_status(flag);
-  }
-  return BSMM_OK;
+  if (total == 0) return BSMM_OK;
+  const bsmm_status s = train(mlp, X, t, n, total, steps, lr, st, missing, limit_ns);
+  if (s != BSMM_OK) return s;
+  // (also when no loss is asked for: a training that was cut short is never taken for a whole one)
+  unsigned flag = 0;
+  if ((final_loss && cudaMemcpyAsync(final_loss, (float*)mlp->grad.p + NP, sizeof(float), cudaMemcpyDeviceToHost, st) !=
+                         cudaSuccess) ||
+      cudaMemcpyAsync(&flag, (unsigned*)mlp->sync.p + 1, sizeof(flag), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return set_error("copy failed"), BSMM_ERR_CUDA;
+  return barrier_status(flag);
 }
 
 }  // namespace

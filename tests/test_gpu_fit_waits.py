@@ -22,14 +22,15 @@ def _fits(n=300):
     return losses
 
 
-def test_barrier_that_runs_out_is_reported():
+@pytest.mark.parametrize("with_loss", [True, False])
+def test_barrier_that_runs_out_is_reported(with_loss):
     import torch
     before = _fits()
     limit = 50_000_000  # 50 ms
     for _ in range(3):
         t0 = time.perf_counter()
         with pytest.raises(P.BsmmError) as ei:
-            P.bsmm_selftest_fit(limit, with_loss=True)
+            P.bsmm_selftest_fit(limit, with_loss=with_loss)
         assert ei.value.status == 4
         assert time.perf_counter() - t0 < 1.0  # one limit, not one per barrier
     torch.cuda.synchronize()
