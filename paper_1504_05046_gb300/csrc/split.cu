@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
   const int CL = a.cl;
   const int cta = blockIdx.x / CL;   // the group: schedules are per group
   const int rank = blockIdx.x % CL;  // this CTA's column block within the group's units
+  grid_wait();  // before anything of global memory is read, the schedule included
   const int ubeg = a.sched_ptr[cta], uend = a.sched_ptr[cta + 1];
 
   if (threadIdx.x == 0) {
@@ -152,7 +153,6 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
-  grid_wait();  // the slices and classes; until here only the plan's own tables were read
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

@@ -235,6 +235,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
   const int CL = a.cl, WCL = CL >> 1;  // column blocks and CTAs of a group
   const int cta = blockIdx.x / WCL;    // the group: schedules are per group
   const int rank = blockIdx.x % WCL;
+  grid_wait();  // before anything of global memory is read, the schedule included
   const int ubeg = a.sched_ptr[cta], uend = a.sched_ptr[cta + 1];
 
   if (threadIdx.x == 0) {
@@ -254,7 +255,6 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
-  grid_wait();  // the slices and classes; until here only the plan's own tables were read
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
