@@ -101,7 +101,8 @@ typedef struct {
                               A plan with groups of 2 or 4, 3 or more slices, a dense block
                               pattern (each pair of column blocks has B tiles at the same
                               inner blocks) and a deep inner sum (3072 elements or so) runs its
-                              own executes with CTAs of two column blocks each: half as many
+                              own executes with CTAs of two column blocks each (unless
+                              store_warps asks for one form or the other): half as many
                               CTAs per group, the same work units, the same result bits. */
   int32_t fp64_tile;       /* FP64 mode: sub-tile edge of a work unit, 32 or 64 (0 = 32) */
   int32_t stages;          /* split modes: depth of the shared-memory ring of 32-deep k chunks
@@ -164,7 +165,8 @@ typedef struct {
                               inner block of q complex elements is 2q real ones deep) and the
                               useful flop count is 8 r c q per nonzero triple. */
   int32_t store_warps;     /* split modes: the contraction kernel's form. 0 = automatic (with
-                              store warps); 2 = with four C store warps (the C store of a
+                              store warps, or two column blocks per CTA, see cluster); 2 = with
+                              four C store warps (the C store of a
                               unit overlaps the next unit's accumulation); 1 = without (the
                               epilogue warps store). Results do not depend on it. An inner
                               block deeper than the exact FP32 accumulation depth (512 for 6

@@ -593,8 +593,9 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   //   356 / 370, 8192: 2651 / 2039; 512 x 131072 deep: 796 / 471
   //   3 slices: 38.5 / 38.6, 60.8 / 71.4, 90.2 / 76.9, 193 / 150, 1398 / 820, 4764 / 2535;
   //   355 / 350, 2622 / 1793; 736 / 370
+  // (not for a plan that asks for C store warps, which the form has none of)
   p->wide = 0;
-  if (CL >= 2 && s >= 3 && p->sw && !p->deep && !base.empty()) {
+  if (CL >= 2 && s >= 3 && p->sw && p->opt.store_warps != 2 && !p->deep && !base.empty()) {
     bool pairs = true;
     for (int cb = 0; cb + 1 < CB && pairs; cb += 2)
       for (int wd = 0; wd < KW && pairs; wd++) pairs = presB[(size_t)cb * KW + wd] == presB[(size_t)(cb + 1) * KW + wd];
