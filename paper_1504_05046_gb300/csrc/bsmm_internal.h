@@ -133,7 +133,8 @@ struct SplitArgs {
   // 1: a plan of its own runs in the 64-column form (wide.cu) with this ring depth; its groups
   // are then of cl/2 CTAs, two column blocks each. pairs (3 and 4 slices): each pair of column
   // blocks is packed slice by slice: a chunk of the pair holds, for every slice, block 2c's
-  // part and then block 2c+1's (bpk_off points at the block's own part of the first slice)
+  // part and then block 2c+1's (bpk_off points at the block's own part of the first slice).
+  // Both are 0 in a batch, which runs the 32-column form and packs block by block
   int32_t wide, wstages, pairs;
   int32_t epi_walk;         // 1: the epilogue finds the accumulation groups on its own k list
                             // (long lists); 0: it takes them from the MMA warps' descriptors
@@ -321,6 +322,7 @@ struct bsmm_plan_s {
   int32_t qmax = 0;          // the largest inner block
   int wide = 0, wstages = 0; // the contraction runs in the 64-column form (SplitArgs::wide)
   int pairs = 0;             // column blocks packed in pairs (SplitArgs::pairs)
+  bsmm::DevBuf d_bpk_off1;   // then also: where they go packed block by block (in a batch)
   int deep = 0;              // some inner block is deeper than the exact FP32 depth
   int64_t Mtot = 0, Ntot = 0, colexp_ld = 0;
   int64_t apk_bytes = 0, bpk_bytes = 0;

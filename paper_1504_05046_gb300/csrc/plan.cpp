@@ -612,16 +612,21 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   p->pairs = p->wide && s <= kWidePairsMaxS;
   cur = 0;
   for (int32_t b : b_blocks) {
-    const int k = b / CB, cb = b % CB;
-    const int64_t bytes = (int64_t)log2i_ceil_div(p->q[k], kSplitKC) * b_chunk_bytes;
-    if (!p->pairs) {
-      bpk_off[b] = cur;
-      cur += bytes;
-    } else if (cb % 2 == 0) {
-      bpk_off[b] = cur;
-      cur += 2 * bytes;
-    } else {  // its partner has the same inner blocks and comes just before it
-      bpk_off[b] = bpk_off[b - 1] + b_chunk_bytes / s;
+    bpk_off[b] = cur;
+    cur += (int64_t)log2i_ceil_div(p->q[b / CB], kSplitKC) * b_chunk_bytes;
+  }
+  std::vector<int64_t> bpk_off1;  // block by block, beside the pairs
+  if (p->pairs) {
+    bpk_off1 = bpk_off;
+    cur = 0;
+    for (int32_t b : b_blocks) {
+      const int k = b / CB, cb = b % CB;
+      if (cb % 2 == 0) {
+        bpk_off[b] = cur;
+        cur += 2 * (int64_t)log2i_ceil_div(p->q[k], kSplitKC) * b_chunk_bytes;
+      } else {  // its partner has the same inner blocks and comes just before it
+        bpk_off[b] = bpk_off[b - 1] + b_chunk_bytes / s;
+      }
     }
   }
   p->bpk_bytes = cur;
@@ -716,6 +721,7 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   if ((st = upload(p->d_presBg, presBg)) != BSMM_OK) return st;
   if ((st = upload(p->d_apk_off, apk_off)) != BSMM_OK) return st;
   if ((st = upload(p->d_bpk_off, bpk_off)) != BSMM_OK) return st;
+  if (p->pairs && (st = upload(p->d_bpk_off1, bpk_off1)) != BSMM_OK) return st;
   if ((st = upload(p->d_a_tiles, a_tiles)) != BSMM_OK) return st;
   if ((st = upload(p->d_b_tiles, b_tiles)) != BSMM_OK) return st;
   if ((st = upload(p->d_a_blocks, a_blocks)) != BSMM_OK) return st;
@@ -834,7 +840,7 @@ void bsmm_destroy(bsmm_plan_t p) {
   if (!p) return;
   DevBuf* bufs[] = {&p->d_r, &p->d_c, &p->d_q, &p->d_ro, &p->d_co, &p->d_kptr, &p->d_klist, &p->d_cs,
                     &p->d_units, &p->d_sched_ptr, &p->d_sched_units, &p->d_row_tile, &p->d_col_tile,
-                    &p->d_presA, &p->d_presB, &p->d_presBg, &p->d_apk_off, &p->d_bpk_off, &p->d_apk, &p->d_bpk,
+                    &p->d_presA, &p->d_presB, &p->d_presBg, &p->d_apk_off, &p->d_bpk_off, &p->d_bpk_off1, &p->d_apk, &p->d_bpk,
                     &p->d_eArow, &p->d_eBcol, &p->d_eAmaxr, &p->d_eBmaxc,
                     &p->d_am, &p->d_bm, &p->d_rowexp, &p->d_colexp, &p->d_urow, &p->d_ucol, &p->d_rowadj, &p->d_coladj, &p->d_emaxr, &p->d_emaxc, &p->d_eA, &p->d_eB, &p->d_a_tiles, &p->d_b_tiles,
                     &p->d_a_blocks, &p->d_b_blocks, &p->d_err, &p->d_timings, &p->d_unit_cta, &p->d_part, &p->d_red};

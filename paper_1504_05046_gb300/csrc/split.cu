@@ -180,15 +180,7 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
         uint8_t* sa = smem + (size_t)stage * STAGE;
         mbar_arrive_expect_tx(&full[stage], STAGE);
         bulk_g2s(sa, cur.asrc + (size_t)cur.kc * A_STAGE, A_STAGE, &full[stage]);
-        bool pairs = false;
-        if constexpr (S <= kWidePairsMaxS) pairs = cur.P->pairs != 0;
-        if (!pairs) {
-          bulk_g2s(sa + A_STAGE, cur.bsrc + (size_t)cur.kc * B_STAGE, B_STAGE, &full[stage]);
-        } else {  // a plan of the 64-column form in a batch: its pairs' slices alternate
-          for (int t = 0; t < S; t++)
-            bulk_g2s(sa + A_STAGE + t * (B_STAGE / S), cur.bsrc + ((size_t)cur.kc * S + t) * (2 * B_STAGE / S),
-                     B_STAGE / S, &full[stage]);
-        }
+        bulk_g2s(sa + A_STAGE, cur.bsrc + (size_t)cur.kc * B_STAGE, B_STAGE, &full[stage]);
         issued |= 1u << stage;
         issued_par = (issued_par & ~(1u << stage)) | (phase << stage);
         if (++stage == stages) {
