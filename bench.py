@@ -38,7 +38,8 @@ PROFILE_FILE = os.path.join(ROOT, "profiles", "split_mma_kernel_nonuniform_dense
 def kernels_per_execute(P, plan, mode, split_scale=0):
     """Kernels one bsmm_execute launches: FP64 the tile kernel; split modes the exponent, pack
     (with the scale classes) and contraction kernels, and with row/column scaling the line
-    scale kernel; plus the split-k reduction when the plan cut a k-list."""
+    scale kernel; plus the split-k reduction when the plan cut a k-list. (With 5 and 6 slices a
+    plan of the 64-column form launches both forms, one of which returns at once: not counted.)"""
     red = int(P.bsmm_plan_ksplit(plan)["n_regions"] > 0)
     return (1 if mode == P.BSMM_FP64 else 3 + int(split_scale)) + red
 

@@ -103,7 +103,11 @@ typedef struct {
                               inner blocks) and a deep inner sum (3072 elements or so) runs its
                               own executes with CTAs of two column blocks each (unless
                               store_warps asks for one form or the other): half as many
-                              CTAs per group, the same work units, the same result bits. */
+                              CTAs per group, the same work units, the same result bits. With
+                              5 and 6 slices that form suits values of one scale and inner
+                              blocks that are deep or of like scale: both forms are launched
+                              and the scales found in the operands decide, at each execute,
+                              which of them runs. */
   int32_t fp64_tile;       /* FP64 mode: sub-tile edge of a work unit, 32 or 64 (0 = 32) */
   int32_t stages;          /* split modes: depth of the shared-memory ring of 32-deep k chunks
                               (k panels in flight), 2..8 and within the 227 KB shared memory of
@@ -534,7 +538,8 @@ bsmm_status bsmm_plan_cost_source(bsmm_plan_t plan, int32_t* source);
  * The contraction launch the planner chose for a plan (host outputs; any may be NULL):
  * cluster = CTAs per column-block group (1, 2 or 4; bsmm_options.cluster = -1 resolved),
  * store_warps = 1 when the kernel form has C store warps (0 also for the form with two column
- * blocks per CTA, see bsmm_options.cluster), epi_walk = 1 when the epilogue
+ * blocks per CTA, which with 5 and 6 slices runs unless the operands' scales speak against it,
+ * see bsmm_options.cluster), epi_walk = 1 when the epilogue
  * walks its own k lists for the accumulation groups (long k lists, 3 to 6 slices with
  * store warps) rather than taking the MMA warps' descriptors, stages = depth of the
  * shared-memory ring, ctas = persistent CTAs (FP64) or groups (split modes) of a launch.

@@ -412,6 +412,7 @@ bsmm_status bsmm_batch_set_args(bsmm_batch_t b, const double* alpha, const void*
       // in one copy (from pairs it took one per slice, about 100 cycles each to issue: four
       // dense products of 2048 to 3072, 3 slices, 1600 us, 1318 block by block).
       b->sargs[i].wide = 0;
+      b->sargs[i].changes = nullptr;
       if (b->sargs[i].pairs) {
         b->sargs[i].pairs = 0;
         b->sargs[i].bpk_off = (const int64_t*)b->plans[i]->d_bpk_off1.p;

@@ -31,6 +31,10 @@ constexpr double kEpiWalkBlocks = 32.0;  // mean k blocks per unit from which th
 constexpr double kWideDepthPairs = 1536.0, kWideDepthMany = 2048.0, kWideDepth = 3072.0;
 constexpr int64_t kWideManyUnits = 8;
 constexpr int kWidePairsMaxS = 4;  // slices up to which that form's column blocks are packed in pairs
+// With more slices that form has one accumulator buffer, and what it gains in so many 32-deep
+// chunks goes into one drain (5 and 6 slices): with the sums in their class's own unit, and at
+// binary positions (see plan.cpp)
+constexpr double kWideDrainPlain[2] = {7.5, 9.5}, kWideDrainPositions[2] = {11.0, 13.5};
 constexpr int kSplitMaxK = 8192;   // inner blocks per product
 constexpr int64_t kSplitMaxInner = int64_t(1) << 22;  // inner elements per product (128-bit sums' headroom)
 
@@ -136,6 +140,13 @@ struct SplitArgs {
   // part and then block 2c+1's (bpk_off points at the block's own part of the first slice).
   // Both are 0 in a batch, which runs the 32-column form and packs block by block
   int32_t wide, wstages, pairs;
+  // 5 and 6 slices: which of the two forms runs depends on the scale classes. changes[0] and
+  // changes[1] count the (row block, k block) and (column block, k block) pairs whose class is
+  // not uniform or not that of the k block before; the 64-column form runs when the share of k
+  // blocks that start a group of their own for that reason is at most max_changes. Null: no
+  // choice (the form is `wide`'s)
+  int32_t* changes;
+  float max_changes;
   int32_t epi_walk;         // 1: the epilogue finds the accumulation groups on its own k list
                             // (long lists); 0: it takes them from the MMA warps' descriptors
   int64_t Mtot, Ntot;
@@ -321,6 +332,8 @@ struct bsmm_plan_s {
   int epi_walk = 0;          // the epilogue walks the k lists itself (SplitArgs::epi_walk)
   int32_t qmax = 0;          // the largest inner block
   int wide = 0, wstages = 0; // the contraction runs in the 64-column form (SplitArgs::wide)
+  float max_changes = 0.0f;  // unless the scale classes change more often (SplitArgs::changes)
+  bsmm::DevBuf d_changes;
   int pairs = 0;             // column blocks packed in pairs (SplitArgs::pairs)
   bsmm::DevBuf d_bpk_off1;   // then also: where they go packed block by block (in a batch)
   int deep = 0;              // some inner block is deeper than the exact FP32 depth

@@ -114,6 +114,8 @@ void fill_split_args(bsmm_plan_s* p, SplitArgs& a, double alpha, const void* A, 
   a.wide = p->wide;
   a.wstages = p->wstages;
   a.pairs = p->pairs;
+  a.changes = (int32_t*)p->d_changes.p;
+  a.max_changes = p->max_changes;
   a.epi_walk = p->epi_walk;
   a.deep = p->deep;
   a.f32 = p->opt.elem == BSMM_F32;

@@ -594,6 +594,17 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   //   3 slices: 38.5 / 38.6, 60.8 / 71.4, 90.2 / 76.9, 193 / 150, 1398 / 820, 4764 / 2535;
   //   355 / 350, 2622 / 1793; 736 / 370
   // (not for a plan that asks for C store warps, which the form has none of)
+  //
+  // Those are values of one scale. With 5 and 6 slices the tensor core waits for every drain,
+  // and an inner block whose scale class differs from its predecessor's is a group of its own:
+  // 6 slices, 3072 x 3072 of 128-row tiles, 4096 deep, classes as they are for U[-1,1] / for
+  // N(0,1) / changing at every inner block, 32-column form against this one:
+  //   inner blocks of 64: 1311 / 1124 us, 1631 / 2044, 2055 / 2617; 128: 1254 / 1052, 1264 /
+  //   1433, 1379 / 1750; 256: 1134 / 1011, 1134 / 1122, 1160 / 1297; 512: 1083 / 990, 1079 /
+  //   998, 1082 / 1058; 5 slices, 128: 1100 / 901, 1108 / 1216, 1195 / 1506
+  // So the choice waits for the data: the slicing counts the changes, both kernels are
+  // launched, and one of them returns at once (3 us). A k block gains in proportion to its
+  // chunks and loses a drain per group; the line lies at kWideDrain* chunks per group.
   p->wide = 0;
   if (CL >= 2 && s >= 3 && p->sw && p->opt.store_warps != 2 && !p->deep && !base.empty()) {
     bool pairs = true;
@@ -606,6 +617,30 @@ bsmm_status plan_split(bsmm_plan_s* p) {
     p->wide = pairs && depth >= (s <= kWidePairsMaxS ? kWideDepthPairs : many ? kWideDepthMany : kWideDepth) ? 1 : 0;
     const int deepest = split_wide_stages(s);
     p->wstages = p->opt.stages ? std::min(p->opt.stages, deepest) : deepest;
+    if (p->wide && s > kWidePairsMaxS) {
+      double chunks = 0.0;
+      for (int32_t k : bk) chunks += log2i_ceil_div(p->q[k], kSplitKC);
+      chunks /= (double)bk.size();
+      const double per_unit = (double)bk.size() / (double)base.size();
+      // groups per k block that the exact depth alone asks for
+      int64_t blocks = 0, groups = 0, fill = maxd + 1;
+      for (int k = 0; k < K; k++) {
+        if (p->q[k] <= 0) continue;
+        blocks++;
+        if (fill + p->q[k] > maxd) groups++, fill = 0;
+        fill += p->q[k];
+      }
+      const double by_depth = (double)groups / (double)blocks;
+      // share f of changes at which f + (1 - f) by_depth groups per k block cost the gain
+      auto limit = [&](double drain) {
+        const double g = chunks / drain;
+        return g < by_depth ? -1.0 : by_depth >= 1.0 ? 1.0 : std::min(1.0, (g - by_depth) / (1.0 - by_depth));
+      };
+      const double most = std::max(limit(kWideDrainPositions[s - 5]),
+                                   std::min(limit(kWideDrainPlain[s - 5]), 1.0 / per_unit));
+      if (most < 0.0) p->wide = 0;
+      p->max_changes = (float)most;
+    }
   }
   // where the column blocks' slices go: block by block, or pair by pair (SplitArgs::pairs; a
   // last block without a partner leaves its partner's place empty)
@@ -757,6 +792,7 @@ bsmm_status plan_split(bsmm_plan_s* p) {
     if ((st = dev_alloc(p->d_eAmaxr, sizeof(int32_t) * std::max<int64_t>(1, Mtot))) != BSMM_OK) return st;
     if ((st = dev_alloc(p->d_eBmaxc, sizeof(int32_t) * std::max<int64_t>(1, Ntot))) != BSMM_OK) return st;
   }
+  if (p->wide && s > kWidePairsMaxS && (st = dev_alloc(p->d_changes, 2 * sizeof(int32_t))) != BSMM_OK) return st;
   if ((st = dev_alloc(p->d_urow, sizeof(int16_t) * std::max<int64_t>(1, (int64_t)K * p->RB))) != BSMM_OK) return st;
   if ((st = dev_alloc(p->d_ucol, sizeof(int16_t) * std::max<int64_t>(1, (int64_t)K * p->CB))) != BSMM_OK) return st;
   if ((st = dev_alloc(p->d_rowadj, sizeof(int16_t) * std::max<int64_t>(1, Mtot))) != BSMM_OK) return st;
@@ -840,7 +876,7 @@ void bsmm_destroy(bsmm_plan_t p) {
   if (!p) return;
   DevBuf* bufs[] = {&p->d_r, &p->d_c, &p->d_q, &p->d_ro, &p->d_co, &p->d_kptr, &p->d_klist, &p->d_cs,
                     &p->d_units, &p->d_sched_ptr, &p->d_sched_units, &p->d_row_tile, &p->d_col_tile,
-                    &p->d_presA, &p->d_presB, &p->d_presBg, &p->d_apk_off, &p->d_bpk_off, &p->d_bpk_off1, &p->d_apk, &p->d_bpk,
+                    &p->d_presA, &p->d_presB, &p->d_presBg, &p->d_apk_off, &p->d_bpk_off, &p->d_bpk_off1, &p->d_changes, &p->d_apk, &p->d_bpk,
                     &p->d_eArow, &p->d_eBcol, &p->d_eAmaxr, &p->d_eBmaxc,
                     &p->d_am, &p->d_bm, &p->d_rowexp, &p->d_colexp, &p->d_urow, &p->d_ucol, &p->d_rowadj, &p->d_coladj, &p->d_emaxr, &p->d_emaxc, &p->d_eA, &p->d_eB, &p->d_a_tiles, &p->d_b_tiles,
                     &p->d_a_blocks, &p->d_b_blocks, &p->d_err, &p->d_timings, &p->d_unit_cta, &p->d_part, &p->d_red};

@@ -93,6 +93,7 @@ constexpr int kExpCluster = 8;  // CTAs of a cluster, at most
 constexpr int kExpResident = 4 * 152;  // CTAs that fill the machine
 __global__ void __launch_bounds__(kExpThreads) split_exp_kernel(const __grid_constant__ SplitArgs a) {
   grid_wait();
+  if (a.changes && blockIdx.x == 0 && threadIdx.x < 2) a.changes[threadIdx.x] = 0;
   const int nz = (int)cluster_size(), z = (int)cluster_rank();
   if (nz > 1) cluster_arrive();  // (waited for before rank 0's shared memory is written: it has started)
   const int b = blockIdx.x / nz;
@@ -194,6 +195,7 @@ template <typename E>
 __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_constant__ SplitArgs a) {
   grid_wait();
   const int b = blockIdx.x;
+  if (a.changes && b == 0 && blockIdx.y == 0 && threadIdx.x < 2) a.changes[threadIdx.x] = 0;
   const bool isA = b < a.n_a_tiles;
   const int t = isA ? a.a_tiles[b] : a.b_tiles[b - a.n_a_tiles];
   int rows, cols;
@@ -463,6 +465,24 @@ __device__ void scale_classes(const SplitArgs& a, ClassShared& sm, int item, int
     if (cls && lane == 0)
       cls[isA ? (int64_t)k * a.RB + b : (int64_t)k * a.CB + b] = (int16_t)(lo > hi ? 0 : lo == hi ? lo - emx : kNonUniform);
   }
+  if (!a.changes) return;
+  // how many of this range's k blocks cannot join the group of the one before (the range's
+  // first one is given the benefit of the doubt): what the choice of the contraction goes by
+  __syncthreads();
+  const int16_t* const cls = isA ? a.urow + b : a.ucol + b;
+  const int64_t ld = isA ? a.RB : a.CB;
+  const uint64_t* const pres = (isA ? a.presA : a.presB) + (int64_t)b * a.kwords;
+  auto present = [&](int k) { return (pres[k >> 6] >> (k & 63) & 1) != 0; };
+  int n = 0;
+  for (int k = k0 + tid; k < k1; k += blockDim.x) {
+    if (!present(k)) continue;
+    int kp = k - 1;
+    while (kp >= k0 && !present(kp)) kp--;
+    const int c = cls[k * ld];
+    if (c == kNonUniform || (kp >= k0 && cls[kp * ld] != c)) n++;
+  }
+  n = __reduce_add_sync(0xffffffffu, n);
+  if (lane == 0 && n) atomicAdd(a.changes + (isA ? 0 : 1), n);
 }
 
 // ---------------------------------------------------------------- kernel 2: slices

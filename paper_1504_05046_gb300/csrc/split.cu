@@ -131,6 +131,8 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
   const int cta = blockIdx.x / CL;   // the group: schedules are per group
   const int rank = blockIdx.x % CL;  // this CTA's column block within the group's units
   grid_wait();  // before anything of global memory is read, the schedule included
+  if constexpr (S > kWidePairsMaxS && SW && !DEEP)
+    if (a.changes && wide_runs(a)) return;
   const int ubeg = a.sched_ptr[cta], uend = a.sched_ptr[cta + 1];
 
   if (threadIdx.x == 0) {
@@ -729,6 +731,8 @@ cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEven
   nvtxRangePushA("bsmm split: contraction");
   after = !ev && split_prep_kernels(a) > 0;
   e = a.wide && !a.prods ? launch_split_wide(a, ctas, st, after) : launch_split_mma(a, ctas, st, after);
+  // the other form, where the scale classes decide between the two
+  if (e == cudaSuccess && a.wide && a.changes && !a.prods) e = launch_split_mma(a, ctas, st, true);
   nvtxRangePop();
   if (ev) cudaEventRecord(ev[++k], st);
   if (e == cudaSuccess && !a.prods && a.n_red > 0) {  // a batch launches its products' reductions
