@@ -289,8 +289,8 @@ void set_error(const std::string& msg);
 void host_release(bsmm_plan_s* p);
 
 // bsmm_plan with an optional donor: a split plan of the same structure and slice count
-// whose slice workspace the new plan shares instead of allocating its own (the packed
-// layout does not depend on the cluster size or the ring depth).
+// whose slice workspace the new plan, made for a batch, shares instead of allocating its own
+// (packed block by block, its size does not depend on the cluster size or the ring depth).
 bsmm_status plan_build(bsmm_plan_t* out, int32_t M, const int32_t* row_sizes, int32_t N, const int32_t* col_sizes,
                        int32_t K, const int32_t* inner_sizes, const uint8_t* a_mask, const uint8_t* b_mask,
                        const uint8_t* c_mask, const bsmm_options* opt, const bsmm_plan_s* donor);

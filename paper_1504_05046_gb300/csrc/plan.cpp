@@ -593,7 +593,8 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   //   356 / 370, 8192: 2651 / 2039; 512 x 131072 deep: 796 / 471
   //   3 slices: 38.5 / 38.6, 60.8 / 71.4, 90.2 / 76.9, 193 / 150, 1398 / 820, 4764 / 2535;
   //   355 / 350, 2622 / 1793; 736 / 370
-  // (not for a plan that asks for C store warps, which the form has none of)
+  // (not for a plan that asks for C store warps, which the form has none of, nor for one that
+  // shares another's workspace: it runs in a batch, in the 32-column form)
   //
   // Those are values of one scale. With 5 and 6 slices the tensor core waits for every drain,
   // and an inner block whose scale class differs from its predecessor's is a group of its own:
@@ -606,7 +607,7 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   // launched, and one of them returns at once (3 us). A k block gains in proportion to its
   // chunks and loses a drain per group; the line lies at kWideDrain* chunks per group.
   p->wide = 0;
-  if (CL >= 2 && s >= 3 && p->sw && p->opt.store_warps != 2 && !p->deep && !base.empty()) {
+  if (CL >= 2 && s >= 3 && p->sw && p->opt.store_warps != 2 && !p->donor && !p->deep && !base.empty()) {
     bool pairs = true;
     for (int cb = 0; cb + 1 < CB && pairs; cb += 2)
       for (int wd = 0; wd < KW && pairs; wd++) pairs = presB[(size_t)cb * KW + wd] == presB[(size_t)(cb + 1) * KW + wd];
@@ -771,7 +772,8 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   p->n_a_blocks = (int32_t)a_blocks.size();
   p->n_b_blocks = (int32_t)b_blocks.size();
   const bsmm_plan_s* d = p->donor;
-  if (d && d->opt.mode != BSMM_FP64 && d->s == p->s && d->apk_bytes == p->apk_bytes && d->bpk_bytes == p->bpk_bytes &&
+  // (a donor whose column blocks are packed in pairs has room for a last one's partner too)
+  if (d && d->opt.mode != BSMM_FP64 && d->s == p->s && d->apk_bytes == p->apk_bytes && d->bpk_bytes >= p->bpk_bytes &&
       d->d_apk.p && d->d_bpk.p) {
     p->d_apk = d->d_apk;
     p->d_bpk = d->d_bpk;
