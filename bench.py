@@ -471,9 +471,10 @@ def timed_steps(plan, run, steps, warmup):
 
 
 def learned_vs_flops(setup, seed, steps, warmup, dev):
-    """The learned schedule against the flop-count schedule on one product: the cost model
-    is trained on unit timings of three other inputs of the same recipe (3 timed runs
-    each, 2000 Adam steps on the GPU), then the product is timed under both schedules.
+    """The learned schedule against the flop-count schedule and the planner's own (by executed
+    work, the default) on one product: the cost model is trained on unit timings of three other
+    inputs of the same recipe (3 timed runs each, 2000 Adam steps on the GPU), then the product
+    is timed under the three schedules.
     `setup(seed, **opt)` plans a product and returns (prob, plan, q, t, run). Returns the
     record, the product's (plan, t, run) under the learned schedule, its timing and the
     clocks sampled while it was timed."""
@@ -490,6 +491,7 @@ def learned_vs_flops(setup, seed, steps, warmup, dev):
     prob, plan, q, t, run = setup(seed, record_timings=1)
     run()
     times = CM.unit_times(plan, run, repeats=3)
+    ms_own, k_own = timed_steps(plan, run, steps, warmup)
     CM.apply_flops(plan)
     ms_flops, k_flops = timed_steps(plan, run, steps, warmup)
     ref = t["C"].clone()
@@ -504,8 +506,10 @@ def learned_vs_flops(setup, seed, steps, warmup, dev):
     y = torch.zeros(len(feats), dtype=torch.float32, device=dev)
     P.bsmm_mlp_predict(mlp, torch.from_numpy(feats).to(dev), y)
     ci = CONTRACTION_INDEX["split"]
-    rec = {"makespan_ms_flop_count": k_flops[ci], "makespan_ms_mlp": k_mlp[ci], "step_ms_flop_count": ms_flops,
-           "step_ms_mlp": ms_mlp, "makespan_gain": 1.0 - k_mlp[ci] / k_flops[ci], "bits_identical": same,
+    rec = {"makespan_ms_flop_count": k_flops[ci], "makespan_ms_default": k_own[ci], "makespan_ms_mlp": k_mlp[ci],
+           "step_ms_flop_count": ms_flops, "step_ms_default": ms_own, "step_ms_mlp": ms_mlp,
+           "makespan_gain": 1.0 - k_mlp[ci] / k_flops[ci], "makespan_gain_over_default": 1.0 - k_mlp[ci] / k_own[ci],
+           "bits_identical": same,
            "train_loss": loss,
            "log_rms_err_flop_count": CM.prediction_error(plan, times, np.maximum(flops, 1.0)),
            "log_rms_err_mlp": CM.prediction_error(plan, times, np.exp(y.cpu().numpy().astype(np.float64))),

@@ -182,7 +182,7 @@ typedef struct {
                               unit's time with it on the GPU and packs the units by those
                               costs (schedule BSMM_SCHED_COSTS). A file that is missing,
                               unreadable, corrupt (checksum), or of another format or feature
-                              version leaves the flop-count costs in place (the fallback);
+                              version leaves the planner's own costs in place (the fallback);
                               bsmm_plan_cost_source tells which was used. The string is read
                               during bsmm_plan only. Results never depend on the schedule. */
 } bsmm_options;
@@ -413,8 +413,8 @@ bsmm_status bsmm_execute_batch(int32_t count, const bsmm_plan_t* plans, const do
  *   forms; FP64: 32 and 64). Writes at most `cap` points to `out` (nullable) and their
  *   total to *count.
  * bsmm_batch_autotune: times the batch (bsmm_batch_set_args called before) under each
- *   candidate: every product is re-planned with that candidate's options (flop-count
- *   schedule; costs set earlier do not carry over), run once to warm up, then `reps`
+ *   candidate: every product is re-planned with that candidate's options (the
+ *   planner's own costs; costs set earlier do not carry over), run once to warm up, then `reps`
  *   times (>= 1) between CUDA events on `stream`; the median is the candidate's time.
  *   Each run writes a scratch C of the caller's C extent, allocated here and freed on
  *   return, so the caller's C is not touched. The batch then keeps its products
@@ -481,8 +481,8 @@ bsmm_status bsmm_batch_autotune_cached(bsmm_batch_t batch, const char* cache_pat
  * 3.2); here work units are packed statically onto persistent CTAs, so the packing
  * needs cost estimates. A small MLP (BSMM_NFEATURES inputs from bsmm_plan_features,
  * two tanh layers of 32, one output = log unit time) is trained on the GPU from
- * measured unit times (bsmm_plan_timings) and its predictions replace the flop-count
- * costs. Results never depend on it (only the order of the units).
+ * measured unit times (bsmm_plan_timings) and its predictions replace the planner's own
+ * costs (BSMM_SCHED_FLOPS). Results never depend on it (only the order of the units).
  *
  * Parameters: one float vector of bsmm_mlp_num_params() entries, in this order:
  * W1[32][F], b1[32], W2[32][32], b2[32], w3[32], b3. Inputs are standardised with the

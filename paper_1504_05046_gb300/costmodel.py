@@ -48,7 +48,8 @@ def apply(plan, mlp):
 
 
 def apply_flops(plan):
-    """Re-pack `plan` with the flop-count costs (the fallback schedule)."""
+    """Re-pack `plan` with its units' useful flop counts as costs (in FP64 mode the planner's own
+    costs; the split modes' are the executed work)."""
     _, flops = bsmm_plan_features(plan)
     bsmm_plan_set_costs(plan, np.maximum(flops, 1.0))
 

@@ -410,7 +410,7 @@ bsmm_status bsmm_batch_set_args(bsmm_batch_t b, const double* alpha, const void*
       b->sargs[i].unit_cta = nullptr;
       // The contraction of a batch is the 32-column form, which takes a column block's slices
       // in one copy (from pairs it took one per slice, about 100 cycles each to issue: four
-      // dense products of 2048 to 3072, 3 slices, 1600 us, 1318 block by block).
+      // dense products of 2048 to 3072, 3 slices, 1600 us, 1190 block by block).
       b->sargs[i].wide = 0;
       b->sargs[i].changes = nullptr;
       if (b->sargs[i].pairs) {

@@ -1050,15 +1050,15 @@ bsmm_status plan_build(bsmm_plan_t* out, int32_t M, const int32_t* row_sizes, in
       return st;
     }
   }
-  // the learned costs of a cost-model file; a file that cannot be used leaves the
-  // flop-count costs (the fallback) and the plan is still built
+  // the learned costs of a cost-model file; a file that cannot be used leaves the planner
+  // its own costs (the fallback) and the plan is still built
   if (!model_path.empty() && o.schedule != BSMM_SCHED_NATURAL && p->n_units > 0) {
     const std::string keep = g_last_error;
     bsmm_mlp_t mlp = nullptr;
     if (bsmm_mlp_load(&mlp, model_path.c_str()) == BSMM_OK) {
       if (bsmm_plan_predict_costs(p, mlp, nullptr) == BSMM_OK) {
         p->cost_source = BSMM_COSTS_MODEL;
-      } else {  // back to the flop-count packing
+      } else {  // back to the planner's own costs
         p->cost = p->unit_cost.empty() ? p->flop_cost : p->unit_cost;
         p->opt.schedule = o.schedule;
         pack_lpt(p);

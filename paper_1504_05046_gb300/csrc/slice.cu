@@ -763,7 +763,6 @@ struct PackLine {
 struct PackEntry {
   int64_t out;    // byte offset of the packed block
   int32_t q, nkc; // inner elements, 32-deep chunks (0: no block)
-  int32_t pass0;  // its first pass
 };
 
 struct PackGrid {
@@ -801,7 +800,7 @@ __global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __gri
     const int en = isA ? 0 : tid >> 5, ln = isA ? tid : tid & 31;
     const int at = isA ? grp : (grp - a.n_a_blocks) * kPackEntries + en;
     PackLine l{-1, 1, 0, 0};
-    PackEntry pe{0, 0, 0, 0};
+    PackEntry pe{0, 0, 0};
     if (isA || at < a.n_b_blocks) {
       const int blk = isA ? a.a_blocks[at] : a.b_blocks[at];
       const int kt = isA ? blk % a.K : blk / a.CB;
