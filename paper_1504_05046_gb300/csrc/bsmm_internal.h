@@ -142,11 +142,17 @@ struct SplitArgs {
   int32_t wide, wstages, pairs;
   // 5 and 6 slices: which of the two forms runs depends on the scale classes. changes[0] and
   // changes[1] count the (row block, k block) and (column block, k block) pairs whose class is
-  // not uniform or not that of the k block before; the 64-column form runs when the share of k
-  // blocks that start a group of their own for that reason is at most max_changes. Null: no
-  // choice (the form is `wide`'s)
+  // not uniform or not that of the k block before, changes[2] the class CTAs that are done; the
+  // last of them chooses the 64-column form (changes[3] = 1) when the share of k blocks that
+  // start a group of their own for that reason is at most max_changes, and gives it its lists
+  // of units, n_groups of them (sched_sel), or empty ones. The 32-column form has a schedule of
+  // its own (sched_ptr2) and looks at changes[3]. Null: no choice (the form is `wide`'s)
   int32_t* changes;
   float max_changes;
+  int32_t n_groups;
+  int32_t* sched_sel;
+  const int32_t* sched_ptr2;
+  const int32_t* sched_units2;
   int32_t epi_walk;         // 1: the epilogue finds the accumulation groups on its own k list
                             // (long lists); 0: it takes them from the MMA warps' descriptors
   int64_t Mtot, Ntot;
@@ -333,7 +339,7 @@ struct bsmm_plan_s {
   int32_t qmax = 0;          // the largest inner block
   int wide = 0, wstages = 0; // the contraction runs in the 64-column form (SplitArgs::wide)
   float max_changes = 0.0f;  // unless the scale classes change more often (SplitArgs::changes)
-  bsmm::DevBuf d_changes;
+  bsmm::DevBuf d_changes, d_sched_ptr2, d_sched_units2, d_sched_sel;
   int pairs = 0;             // column blocks packed in pairs (SplitArgs::pairs)
   bsmm::DevBuf d_bpk_off1;   // then also: where they go packed block by block (in a batch)
   int deep = 0;              // some inner block is deeper than the exact FP32 depth

@@ -116,6 +116,10 @@ void fill_split_args(bsmm_plan_s* p, SplitArgs& a, double alpha, const void* A, 
   a.pairs = p->pairs;
   a.changes = (int32_t*)p->d_changes.p;
   a.max_changes = p->max_changes;
+  a.n_groups = p->ctas;
+  a.sched_sel = (int32_t*)p->d_sched_sel.p;
+  a.sched_ptr2 = (const int32_t*)p->d_sched_ptr2.p;
+  a.sched_units2 = (const int32_t*)p->d_sched_units2.p;
   a.epi_walk = p->epi_walk;
   a.deep = p->deep;
   a.f32 = p->opt.elem == BSMM_F32;

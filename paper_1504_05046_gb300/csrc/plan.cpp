@@ -245,11 +245,13 @@ inline int log2i_ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b);
 
 inline float lg(double x) { return (float)std::log2(1.0 + x); }
 
-void pack_lpt(bsmm_plan_s* p) {
+void pack_bins(const bsmm_plan_s* p, int bins, std::vector<int32_t>& ptr, std::vector<int32_t>& units) {
   std::vector<int64_t> seg;
-  wave_segments(0, (int64_t)p->cost.size(), p->ctas, seg);
-  lpt_pack(p->cost, p->ctas, p->opt.schedule == BSMM_SCHED_NATURAL, p->sched_ptr, p->sched_units, &seg);
+  wave_segments(0, (int64_t)p->cost.size(), bins, seg);
+  lpt_pack(p->cost, bins, p->opt.schedule == BSMM_SCHED_NATURAL, ptr, units, &seg);
 }
+
+void pack_lpt(bsmm_plan_s* p) { pack_bins(p, p->ctas, p->sched_ptr, p->sched_units); }
 
 int default_ctas(const bsmm_plan_s* p) { return default_bins(p); }
 
@@ -257,6 +259,14 @@ bsmm_status upload_schedule(bsmm_plan_s* p) {
   bsmm_status st;
   if ((st = upload(p->d_sched_ptr, p->sched_ptr)) != BSMM_OK) return st;
   if ((st = upload(p->d_sched_units, p->sched_units)) != BSMM_OK) return st;
+  if (p->wide && p->s > kWidePairsMaxS) {
+    // the 32-column form, should the data choose it: half as many groups, of twice the CTAs
+    std::vector<int32_t> ptr, units;
+    pack_bins(p, (p->ctas + 1) / 2, ptr, units);
+    if ((st = upload(p->d_sched_ptr2, ptr)) != BSMM_OK) return st;
+    if ((st = upload(p->d_sched_units2, units)) != BSMM_OK) return st;
+    if ((st = upload(p->d_sched_sel, p->sched_ptr)) != BSMM_OK) return st;
+  }
   return BSMM_OK;
 }
 
@@ -604,7 +614,7 @@ bsmm_status plan_split(bsmm_plan_s* p) {
   //   1433, 1379 / 1750; 256: 1134 / 1011, 1134 / 1122, 1160 / 1297; 512: 1083 / 990, 1079 /
   //   998, 1082 / 1058; 5 slices, 128: 1100 / 901, 1108 / 1216, 1195 / 1506
   // So the choice waits for the data: the slicing counts the changes, both kernels are
-  // launched, and one of them returns at once (3 us). A k block gains in proportion to its
+  // launched, and one of them has nothing to do (3 us). A k block gains in proportion to its
   // chunks and loses a drain per group; the line lies at kWideDrain* chunks per group.
   p->wide = 0;
   if (CL >= 2 && s >= 3 && p->sw && p->opt.store_warps != 2 && !p->donor && !p->deep && !base.empty()) {
@@ -794,7 +804,7 @@ bsmm_status plan_split(bsmm_plan_s* p) {
     if ((st = dev_alloc(p->d_eAmaxr, sizeof(int32_t) * std::max<int64_t>(1, Mtot))) != BSMM_OK) return st;
     if ((st = dev_alloc(p->d_eBmaxc, sizeof(int32_t) * std::max<int64_t>(1, Ntot))) != BSMM_OK) return st;
   }
-  if (p->wide && s > kWidePairsMaxS && (st = dev_alloc(p->d_changes, 2 * sizeof(int32_t))) != BSMM_OK) return st;
+  if (p->wide && s > kWidePairsMaxS && (st = dev_alloc(p->d_changes, 4 * sizeof(int32_t))) != BSMM_OK) return st;
   if ((st = dev_alloc(p->d_urow, sizeof(int16_t) * std::max<int64_t>(1, (int64_t)K * p->RB))) != BSMM_OK) return st;
   if ((st = dev_alloc(p->d_ucol, sizeof(int16_t) * std::max<int64_t>(1, (int64_t)K * p->CB))) != BSMM_OK) return st;
   if ((st = dev_alloc(p->d_rowadj, sizeof(int16_t) * std::max<int64_t>(1, Mtot))) != BSMM_OK) return st;
@@ -878,7 +888,7 @@ void bsmm_destroy(bsmm_plan_t p) {
   if (!p) return;
   DevBuf* bufs[] = {&p->d_r, &p->d_c, &p->d_q, &p->d_ro, &p->d_co, &p->d_kptr, &p->d_klist, &p->d_cs,
                     &p->d_units, &p->d_sched_ptr, &p->d_sched_units, &p->d_row_tile, &p->d_col_tile,
-                    &p->d_presA, &p->d_presB, &p->d_presBg, &p->d_apk_off, &p->d_bpk_off, &p->d_bpk_off1, &p->d_changes, &p->d_apk, &p->d_bpk,
+                    &p->d_presA, &p->d_presB, &p->d_presBg, &p->d_apk_off, &p->d_bpk_off, &p->d_bpk_off1, &p->d_changes, &p->d_sched_ptr2, &p->d_sched_units2, &p->d_sched_sel, &p->d_apk, &p->d_bpk,
                     &p->d_eArow, &p->d_eBcol, &p->d_eAmaxr, &p->d_eBmaxc,
                     &p->d_am, &p->d_bm, &p->d_rowexp, &p->d_colexp, &p->d_urow, &p->d_ucol, &p->d_rowadj, &p->d_coladj, &p->d_emaxr, &p->d_emaxc, &p->d_eA, &p->d_eB, &p->d_a_tiles, &p->d_b_tiles,
                     &p->d_a_blocks, &p->d_b_blocks, &p->d_err, &p->d_timings, &p->d_unit_cta, &p->d_part, &p->d_red};
@@ -1050,8 +1060,8 @@ bsmm_status plan_build(bsmm_plan_t* out, int32_t M, const int32_t* row_sizes, in
       return st;
     }
   }
-  // the learned costs of a cost-model file; a file that cannot be used leaves the planner
-  // its own costs (the fallback) and the plan is still built
+  // the learned costs of a cost-model file; a file that cannot be used leaves the
+  // planner's own (the fallback) and the plan is still built
   if (!model_path.empty() && o.schedule != BSMM_SCHED_NATURAL && p->n_units > 0) {
     const std::string keep = g_last_error;
     bsmm_mlp_t mlp = nullptr;

@@ -93,7 +93,7 @@ constexpr int kExpCluster = 8;  // CTAs of a cluster, at most
 constexpr int kExpResident = 4 * 152;  // CTAs that fill the machine
 __global__ void __launch_bounds__(kExpThreads) split_exp_kernel(const __grid_constant__ SplitArgs a) {
   grid_wait();
-  if (a.changes && blockIdx.x == 0 && threadIdx.x < 2) a.changes[threadIdx.x] = 0;
+  if (a.changes && blockIdx.x == 0 && threadIdx.x < 3) a.changes[threadIdx.x] = 0;
   const int nz = (int)cluster_size(), z = (int)cluster_rank();
   if (nz > 1) cluster_arrive();  // (waited for before rank 0's shared memory is written: it has started)
   const int b = blockIdx.x / nz;
@@ -195,7 +195,7 @@ template <typename E>
 __global__ void __launch_bounds__(256) split_exp_lines_kernel(const __grid_constant__ SplitArgs a) {
   grid_wait();
   const int b = blockIdx.x;
-  if (a.changes && b == 0 && blockIdx.y == 0 && threadIdx.x < 2) a.changes[threadIdx.x] = 0;
+  if (a.changes && b == 0 && blockIdx.y == 0 && threadIdx.x < 3) a.changes[threadIdx.x] = 0;
   const bool isA = b < a.n_a_tiles;
   const int t = isA ? a.a_tiles[b] : a.b_tiles[b - a.n_a_tiles];
   int rows, cols;
@@ -367,9 +367,10 @@ struct ClassShared {
   int32_t tile[kSplitBM];  // the lines' tiles
   int32_t em[kSplitBM];    // and largest exponents
   uint32_t first[kSplitBM / 32];  // bit: the line is the first of its tile here
+  int last;                // this CTA is the last one done
 };
 
-__device__ void scale_classes(const SplitArgs& a, ClassShared& sm, int item, int nr) {
+__device__ void scale_classes(const SplitArgs& a, ClassShared& sm, int item, int nr, int items) {
   const int blk = item / nr;
   const bool isA = blk < a.RB;
   const int b = isA ? blk : blk - a.RB;
@@ -483,6 +484,17 @@ __device__ void scale_classes(const SplitArgs& a, ClassShared& sm, int item, int
   }
   n = __reduce_add_sync(0xffffffffu, n);
   if (lane == 0 && n) atomicAdd(a.changes + (isA ? 0 : 1), n);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) sm.last = atomicAdd(a.changes + 2, 1) == items - 1;
+  __syncthreads();
+  if (!sm.last) return;
+  // the choice, made once for both kernels
+  __threadfence();
+  const float fa = (float)__ldcg(a.changes) / (float)a.n_a_blocks, fb = (float)__ldcg(a.changes + 1) / (float)a.n_b_blocks;
+  const bool wide = 1.0f - (1.0f - fa) * (1.0f - fb) <= a.max_changes;
+  if (tid == 0) a.changes[3] = wide;
+  for (int g = tid; g <= a.n_groups; g += blockDim.x) a.sched_sel[g] = wide ? a.sched_ptr[g] : 0;
 }
 
 // ---------------------------------------------------------------- kernel 2: slices
@@ -783,7 +795,7 @@ __global__ void __launch_bounds__(kPackThreads, 3) split_pack_kernel(const __gri
   grid_wait();
   const int turn = blockIdx.x / g.every;  // every g.every-th CTA: offsets and scale classes
   if (turn < g.ncls && blockIdx.x % g.every == 0) {
-    scale_classes(a, sm.cls, turn, g.ranges);
+    scale_classes(a, sm.cls, turn, g.ranges, g.ncls);
     return;
   }
   auto& lines = sm.pk.lines;

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(threads_of<SW>(), 1) split_mma_kernel(const __
   const int rank = blockIdx.x % CL;  // this CTA's column block within the group's units
   grid_wait();  // before anything of global memory is read, the schedule included
   if constexpr (S > kWidePairsMaxS && SW && !DEEP)
-    if (a.changes && wide_runs(a)) return;
+    if (a.changes && a.changes[3]) return;  // the 64-column form ran
   const int ubeg = a.sched_ptr[cta], uend = a.sched_ptr[cta + 1];
 
   if (threadIdx.x == 0) {
@@ -730,9 +730,16 @@ cudaError_t launch_split(const SplitArgs& a, int ctas, cudaStream_t st, cudaEven
   if (e != cudaSuccess) return e;
   nvtxRangePushA("bsmm split: contraction");
   after = !ev && split_prep_kernels(a) > 0;
-  e = a.wide && !a.prods ? launch_split_wide(a, ctas, st, after) : launch_split_mma(a, ctas, st, after);
-  // the other form, where the scale classes decide between the two
-  if (e == cudaSuccess && a.wide && a.changes && !a.prods) e = launch_split_mma(a, ctas, st, true);
+  if (a.wide && !a.prods && a.changes) {  // both forms, of which the scale classes chose one
+    SplitArgs b = a;
+    b.sched_ptr = a.sched_sel;
+    e = launch_split_wide(b, ctas, st, after);
+    b.sched_ptr = a.sched_ptr2;
+    b.sched_units = a.sched_units2;
+    if (e == cudaSuccess) e = launch_split_mma(b, (ctas + 1) / 2, st, true);
+  } else {
+    e = a.wide && !a.prods ? launch_split_wide(a, ctas, st, after) : launch_split_mma(a, ctas, st, after);
+  }
   nvtxRangePop();
   if (ev) cudaEventRecord(ev[++k], st);
   if (e == cudaSuccess && !a.prods && a.n_red > 0) {  // a batch launches its products' reductions

@@ -695,13 +695,6 @@ __device__ __forceinline__ bool scale_class(const SplitArgs& P, int k, int rb, i
   return true;
 }
 
-// Whether the 64-column form runs, of the two that were launched (a.changes): both kernels
-// come to the same answer.
-__device__ __forceinline__ bool wide_runs(const SplitArgs& a) {
-  const float fa = (float)a.changes[0] / (float)a.n_a_blocks, fb = (float)a.changes[1] / (float)a.n_b_blocks;
-  return 1.0f - (1.0f - fa) * (1.0f - fb) <= a.max_changes;
-}
-
 struct GroupRule {
   bool uni;
   int sig, depth, kdepth;

@@ -13,9 +13,11 @@
 // The price: two accumulator buffers of S x 64 columns fit TMEM only up to 4 slices. With 5
 // and 6 there is one, and the tensor core waits while a group is drained (3200 cycles of a
 // 26000-cycle group of the dense product, 6000 at binary positions), so the form suits
-// products whose groups are long: with those slice counts the 32-column form is launched
-// behind this one, and by the scale classes that the slicing counted one of the two returns at
-// once (wide_runs; the limit is plan.cpp's); and the 128-bit sums of 64 columns take 128 registers of each of the 8 epilogue warps, which
+// products whose groups are long. With those slice counts the 32-column form is launched
+// behind this one, and one of the two has nothing to do (3 us), chosen from the scale classes
+// by the slicing (slice.cu; the limit is plan.cpp's). This kernel finds its lists empty then: a
+// test and a return at its top cost it 0.5% (dense 4096: 1948 against 1938 us).
+// And the 128-bit sums of 64 columns take 128 registers of each of the 8 epilogue warps, which
 // leaves no room for store warps: the epilogue stores a unit itself while the next unit's
 // first group runs.
 // Contraction, 32-column form against this one: dense 16384, 6 slices, 133.1 to 112.3 ms
@@ -25,10 +27,8 @@
 //
 // Roles: warp 0 producer, warps 1 and 2 MMA issue, warp 3 idle, warps 4 to 11 epilogue. The
 // unit list, the k lists, the accumulation groups and the exact sums are those of the
-// 32-column form with groups of 2 or 4 CTAs: a plan's units and its schedule are the same for
-// both (a batch runs them with the 32-column form), and so are the result bits. As the second
-// of the two the 32-column form has twice as many groups as are resident at once; it takes 1%
-// to 2% longer than with a schedule of its own.
+// 32-column form with groups of 2 or 4 CTAs: a plan's units are the same for both (a batch
+// runs them with the 32-column form), and so are the result bits.
 #include <cstdint>
 #include <type_traits>
 
@@ -240,8 +240,6 @@ __global__ void __launch_bounds__(kWideThreads, 1) split_mma_wide_kernel(const _
   const int cta = blockIdx.x / WCL;    // the group: schedules are per group
   const int rank = blockIdx.x % WCL;
   grid_wait();  // before anything of global memory is read, the schedule included
-  if constexpr (NB == 1)
-    if (a.changes && !wide_runs(a)) return;
   const int ubeg = a.sched_ptr[cta], uend = a.sched_ptr[cta + 1];
 
   if (threadIdx.x == 0) {
