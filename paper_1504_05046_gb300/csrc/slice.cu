@@ -521,10 +521,12 @@ __device__ void scale_classes(const SplitArgs& a, ClassShared& sm, int item, int
 // levels fit a 32-bit word (p = 2, 9, 16); the next three are those of V >> 21, whose
 // dropped bits are the same in both remainders.
 //
-// What bounds it: HBM (8 bytes read and 2S written per element): 16384 dense, six slices,
-// 10.7 GB in 1.96 ms (5.5 TB/s), where significand windows with variable rounding per level
-// took 2.92 ms (integer pipe 80% busy, DRAM 43%, and each block's chunks one after the
-// other with nothing in flight between them). float32 8192, four slices: 0.62 to 0.45 ms.
+// What bounds it: HBM (8 bytes read and 2S written per element) and the integer pipe
+// together: 16384 dense, six slices, 10.7 GB in 1.96 to 2.02 ms (5.4 TB/s); on 6144 DRAM is
+// 64% busy and the integer pipe 79% (per instruction issued 2.2 warps wait for data, 1.4 for
+// the pipe). Before, significand windows with variable rounding per level took 2.92 ms
+// (integer pipe 80% busy, DRAM 43%, and each block's chunks one after the other with nothing
+// in flight between them). float32 8192, four slices: 0.62 to 0.45 ms.
 template <typename T>
 struct Slice2;  // two slices' values in one word; times the elements' signs
 template <>
